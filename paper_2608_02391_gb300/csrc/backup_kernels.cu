@@ -29,28 +29,10 @@ __device__ __forceinline__ uint2 pack4(const float v[4]) {
   return make_uint2(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]));
 }
 
-// Validated tile bounds: false (and a flag) for a tile outside the arena.
-__device__ __forceinline__ bool backup_tile(const uint64_t *tiles, uint64_t t, uint64_t n_alloc,
-                                            uint64_t &b, uint64_t &e) {
-  b = tiles[2 * t];
-  e = tiles[2 * t + 1];
-  if (b > e || e > n_alloc || e - b > (uint64_t)COPES_TILE_MAX) {
-    if (threadIdx.x == 0) backup_flag(kErrTileRange);
-    return false;
-  }
-  return true;
-}
-
-// One block per tile; thread-strided 4-element groups.
+// Thread-strided 4-element groups of the elements [b, e).
 template <int OP>
-__global__ void __launch_bounds__(kThreads) backup_elem_kernel(const __grid_constant__ ElemArgs a,
-                                                               uint16_t *backup) {
-  uint64_t b, e;
-  if (!backup_tile(a.tiles, blockIdx.x, a.n_alloc, b, e)) return;
-  if (OP == kBackupPerturbPair && (b < a.partner_base || e - a.partner_base > a.partner_len)) {
-    if (threadIdx.x == 0) backup_flag(kErrPartnerRange);
-    return;
-  }
+__device__ __forceinline__ void backup_elem_stretch(const ElemArgs &a, uint16_t *backup, const SlimTable &tab,
+                                                    uint64_t b, uint64_t e) {
   constexpr bool kPerturb = OP == kBackupPerturb || OP == kBackupPerturbPair;
   uint16_t *w = static_cast<uint16_t *>(a.w);
   // partner element g at pw[g - partner_base]; partner_base is a multiple of 4 and at most b,
@@ -75,14 +57,17 @@ __global__ void __launch_bounds__(kThreads) backup_elem_kernel(const __grid_cons
     } else {
       for (int k = 0; k < 4; ++k) th[k] = (g4 + k >= b && g4 + k < e) ? bf16_to_f32(backup[g4 + k]) : 0.0f;
     }
-    uint32_t x[4];
-    philox4x32_10_rk((uint32_t)(g4 >> 2), (uint32_t)(g4 >> 34), 0u, COPES_TAG_NOISE, a.rk, x);
-    float xn[4], r[4], v[4], vp[4];
-    normal_parts4_x2(x, a.coeffs.central2, a.coeffs.tail, xn, r);  // r = s sigma R(L)
+    uint32_t x[1][4];
+    philox4x32_10_rk((uint32_t)(g4 >> 2), (uint32_t)(g4 >> 34), 0u, COPES_TAG_NOISE, a.rk, x[0]);
+    unsigned long long e2[1][2];
+    normals_packed<1>(x, tab, e2);
+    float eps[4], v[4], vp[4];
+    unpack_f32x2(e2[0][0], eps[0], eps[1]);
+    unpack_f32x2(e2[0][1], eps[2], eps[3]);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      v[k] = __fmaf_rn(r[k], xn[k], th[k]);
-      vp[k] = __fmaf_rn(-r[k], xn[k], th[k]);
+      v[k] = __fmaf_rn(a.a, eps[k], th[k]);
+      vp[k] = __fmaf_rn(-a.a, eps[k], th[k]);
     }
     if (full) {
       *reinterpret_cast<uint2 *>(w + g4) = pack4(v);
@@ -97,18 +82,32 @@ __global__ void __launch_bounds__(kThreads) backup_elem_kernel(const __grid_cons
   }
 }
 
+template <int OP>
+__global__ void __launch_bounds__(kThreads) backup_elem_kernel(const __grid_constant__ ElemArgs a,
+                                                               uint16_t *backup) {
+  constexpr bool kPerturb = OP == kBackupPerturb || OP == kBackupPerturbPair;
+  __shared__ __align__(16) float4 s_tab[kPerturb ? SlimTable::kFloat4s : 1];
+  if (kPerturb) SlimTable::fill(s_tab);
+  __syncthreads();
+  const SlimTable tab(s_tab);
+  for_unit(blockIdx.x, a.units, a.tiles, a.n_tiles, a.n_alloc, backup_flag, [&](uint64_t b, uint64_t e) {
+    if (OP != kBackupPerturbPair || (b >= a.partner_base && e - a.partner_base <= a.partner_len)) return true;
+    backup_flag(kErrPartnerRange);
+    return false;
+  }, [&](uint64_t b, uint64_t e) { backup_elem_stretch<OP>(a, backup, tab, b, e); });
+}
+
 // The update: all P noise vectors regenerated per group in registers (noise_sum_groups,
 // the tile update's loop), the backup read only after the noise loop, the new context
 // written to both copies.  Same launch shape as the tile update: G groups per thread,
-// 4 resident blocks per SM.
-template <int G, bool HI0>
-__device__ __forceinline__ void backup_update_tile(const UpdateArgs &a, uint16_t *backup, const float *s_w,
-                                                   const uint32_t (*s_rk)[20], const uint32_t (*s_fk)[20],
-                                                   uint64_t b, uint64_t e) {
+// 4 resident blocks per SM.  All counters of [b, e) have the high word s.q_hi.
+template <int G>
+__device__ __forceinline__ void backup_update_range(const UpdateArgs &a, uint16_t *backup, const UpdateSmem &s,
+                                                    uint64_t b, uint64_t e) {
   uint16_t *w = static_cast<uint16_t *>(a.w);
   for (uint64_t base = (b & ~3ull) + 4ull * threadIdx.x; base < e; base += 4ull * kThreads * G) {
     float acc[G][4];
-    noise_sum_groups<G, HI0>(base, a.n_noise, s_w, s_rk, s_fk, acc);
+    noise_sum_groups<G>(base, a.n_noise, s, acc);
 #pragma unroll
     for (int i = 0; i < G; ++i) {
       const uint64_t g4 = base + 4ull * kThreads * i;
@@ -139,19 +138,27 @@ constexpr int kBackupUpdateBlocksPerSM = 4;
 
 __global__ void __launch_bounds__(kThreads, kBackupUpdateBlocksPerSM)
     backup_update_kernel(const __grid_constant__ UpdateArgs a, uint16_t *backup) {
-  __shared__ float s_w[COPES_MAX_NOISE];
-  __shared__ __align__(16) uint32_t s_rk[COPES_MAX_NOISE][20];
-  __shared__ __align__(16) uint32_t s_fk[COPES_MAX_NOISE][20];
-  noise_weights_to_smem(a, s_w, s_rk, s_fk);
-  uint64_t b, e;
-  if (!backup_tile(a.tiles, blockIdx.x, a.n_alloc, b, e)) return;
-  if ((e >> 34) == 0) backup_update_tile<kBackupUpdateGroups, true>(a, backup, s_w, s_rk, s_fk, b, e);
-  else backup_update_tile<kBackupUpdateGroups, false>(a, backup, s_w, s_rk, s_fk, b, e);
+  extern __shared__ __align__(128) char s_update[];
+  __shared__ UnitSmem s_unit;
+  if (threadIdx.x == 0) units_init(s_unit);
+  UpdateSmem s = update_prologue(a, s_update);  // ends with __syncthreads
+  for_units(s_unit, a.units, backup_flag, [&](uint32_t unit, NextUnit &) {
+    for_unit(unit, a.units, a.tiles, a.n_tiles, a.n_alloc, backup_flag, [](uint64_t, uint64_t) { return true; },
+             [&](uint64_t b, uint64_t e) {
+      while (b < e) {  // one pass, two where the counters' high word changes
+        const uint64_t end = min(e, ((b >> 34) + 1) << 34);
+        update_keys_for(a, s, b);
+        backup_update_range<kBackupUpdateGroups>(a, backup, s, b, end);
+        b = end;
+      }
+    });
+  });
 }
 
-cudaError_t launch_backup_elementwise(int op, const ElemArgs &a, uint16_t *backup, cudaStream_t s) {
+cudaError_t launch_backup_elementwise(int op, ElemArgs &a, uint16_t *backup, cudaStream_t s) {
   if (a.n_tiles == 0) return cudaSuccess;
-  const unsigned grid = (unsigned)a.n_tiles;
+  a.units = plan_tile_units(a.n_tiles, a.n_alloc, 2, 1216);
+  const unsigned grid = a.units.n_units;
   switch (op) {
     case kBackupSave: backup_elem_kernel<kBackupSave><<<grid, kThreads, 0, s>>>(a, backup); break;
     case kBackupPerturb: backup_elem_kernel<kBackupPerturb><<<grid, kThreads, 0, s>>>(a, backup); break;
@@ -161,9 +168,10 @@ cudaError_t launch_backup_elementwise(int op, const ElemArgs &a, uint16_t *backu
   return cudaGetLastError();
 }
 
-cudaError_t launch_backup_update(const UpdateArgs &a, uint16_t *backup, cudaStream_t s) {
+cudaError_t launch_backup_update(UpdateArgs &a, uint16_t *backup, cudaStream_t s) {
   if (a.n_tiles == 0) return cudaSuccess;
-  backup_update_kernel<<<(unsigned)a.n_tiles, kThreads, 0, s>>>(a, backup);
+  a.units = plan_tile_units(a.n_tiles, a.n_alloc, 3, 608);
+  backup_update_kernel<<<a.units.n_units, kThreads, update_smem_bytes(a.n_noise), s>>>(a, backup);
   return cudaGetLastError();
 }
 

@@ -9,61 +9,18 @@
 
 namespace copes {
 
+__device__ __forceinline__ uint32_t smem_addr(const void *p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+
 __device__ __forceinline__ float lg2_approx(float x) {
   float y;
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 
-__device__ __forceinline__ float sqrt_approx(float x) {
-  float y;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-template <int N>
-__device__ __forceinline__ float horner(const float (&c)[N], float v) {
-  // Horner's rule, highest coefficient first
-  float r = c[N - 1];
-#pragma unroll
-  for (int i = N - 2; i >= 0; --i) r = __fmaf_rn(r, v, c[i]);
-  return r;
-}
-
-// Standard normal from one Philox word w: eps = Phi^-1(u), u = ((w & 0x7FFFFE) | 1) 2^-23.
-// OR-ing those bits (made odd) under the exponent of 2 gives the float 2 + m 2^-22 with m
-// odd, so x = 2u - 1 = that - 3 is exact in one add.  Then
-//   eps = sqrt(2) erfinv(x) = x * R(L),  L = log2(1 - x^2),
-// with R a fitted polynomial in L on the central range and in sqrt(-L) - shift on the tail
-// (coefficients: normal_coeffs.h).  R is evaluated relative to its own value, so eps has
-// a small relative error for every x, including x near 0 (L -> 0) and near +-1.
-//
-// The parts return x and r = scale * R(L) when given coefficients pre-multiplied by
-// scale, so a caller forms scale * eps + b as one fma(r, x, b).
-__device__ __forceinline__ float lattice_x(uint32_t w) {
-  return __fadd_rn(__uint_as_float((w & 0x007FFFFEu) | 0x40000001u), -3.0f);
-}
-
-template <int NT>
-__device__ __forceinline__ float tail_ratio(const float (&tail)[NT], float L) {
-  return horner(tail, __fadd_rn(sqrt_approx(-L), -COPES_NORMAL_TAIL_SHIFT));
-}
-
-// One word.  The tail polynomial runs only when some active lane needs it.
-template <int NC, int NT>
-__device__ __forceinline__ void normal_parts(uint32_t w, const float (&central)[NC],
-                                             const float (&tail)[NT], float &x, float &r) {
-  x = lattice_x(w);
-  const float L = lg2_approx(__fmaf_rn(-x, x, 1.0f));
-  r = horner(central, L);
-  const bool in_tail = L < COPES_NORMAL_L_SPLIT;
-  if (__any_sync(__activemask(), in_tail)) {
-    if (in_tail) r = tail_ratio(tail, L);
-  }
-}
-
-// Packed fp32 pairs: one fma.rn.f32x2 performs the two lanes' fp32 fmas, each rounded
-// exactly as a scalar fma, at half the instruction count.
+// Packed fp32 pairs: one instruction performs the two lanes' fp32 operations, each rounded
+// exactly as the scalar one, at half the instruction count.
 __device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi) {
   unsigned long long r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
@@ -78,49 +35,6 @@ __device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, un
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
-
-// The four words of one Philox block: normal_parts for each, with the central polynomial
-// evaluated on two packed pairs (central2 holds each coefficient twice, (c, c); the same
-// results bit for bit) and a single warp vote for the tail (taken by a warp with
-// probability ~6%), so the common path carries no per-normal branch.
-template <int NC, int NT>
-__device__ __forceinline__ void normal_parts4_x2(const uint32_t (&w)[4],
-                                                 const unsigned long long (&central2)[NC],
-                                                 const float (&tail)[NT], float (&x)[4],
-                                                 float (&r)[4]) {
-  float L[4];
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    x[e] = lattice_x(w[e]);
-    L[e] = lg2_approx(__fmaf_rn(-x[e], x[e], 1.0f));
-  }
-#pragma unroll
-  for (int p = 0; p < 2; ++p) {
-    const unsigned long long Lp = pack_f32x2(L[2 * p], L[2 * p + 1]);
-    unsigned long long acc = central2[NC - 1];
-#pragma unroll
-    for (int i = NC - 2; i >= 0; --i) acc = fma_f32x2(acc, Lp, central2[i]);
-    unpack_f32x2(acc, r[2 * p], r[2 * p + 1]);
-  }
-  const float L_min = fminf(fminf(L[0], L[1]), fminf(L[2], L[3]));
-  if (__any_sync(__activemask(), L_min < COPES_NORMAL_L_SPLIT)) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-      if (L[e] < COPES_NORMAL_L_SPLIT) r[e] = tail_ratio(tail, L[e]);
-  }
-}
-
-#define COPES_UNIT_COEFFS                                                                     \
-  constexpr float unit_central[COPES_NORMAL_CENTRAL_DEGREE + 1] = COPES_NORMAL_CENTRAL_COEFFS; \
-  constexpr float unit_tail[COPES_NORMAL_TAIL_DEGREE + 1] = COPES_NORMAL_TAIL_COEFFS
-
-__device__ __forceinline__ float normal_from_word(uint32_t w) {
-  COPES_UNIT_COEFFS;
-  float x, r;
-  normal_parts(w, unit_central, unit_tail, x, r);
-  return __fmul_rn(x, r);
-}
-
 __device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b) {
   unsigned long long d;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
@@ -136,158 +50,115 @@ __device__ __forceinline__ unsigned long long splat_f32x2(float c) {
   return (b << 32) | b;
 }
 
-// The normals of G Philox blocks with a single warp vote for the tail, every step on packed
-// fp32 pairs with compile-time coefficients: each block's central polynomial, then, only
-// when some lane of the warp holds a word in the tail, the tail polynomial for those words.  x2[i][p] = (x_2p, x_2p+1) and r2[i][p] = (r_2p, r_2p+1) of
-// block i, eps = x * r.  Each packed op rounds like its scalar form and x^2 - 1 is the
-// exact negative of 1 - x^2 under round-to-nearest, so each eps is normal_from_word of its
-// word bit for bit, with one vote for G blocks instead of one per word.
-template <int G>
-__device__ __forceinline__ void normal_parts_groups_packed(const uint32_t (&w)[G][4],
-                                                           unsigned long long (&x2)[G][2],
-                                                           unsigned long long (&r2)[G][2]) {
-  COPES_UNIT_COEFFS;
-  float L[G][4];
-  float L_min = 0.0f;
+// ---------------------------------------------------------------- word -> normal
+// Standard normal from one Philox word w: eps = Phi^-1(u), u = ((w & 0x7FFFFE) | 1) 2^-23.
+// OR-ing those bits (made odd) under the exponent of 2 gives the float 2 + m 2^-22 with m
+// odd, so x = 2u - 1 = that - 3 is exact in one add.  Then
+//   eps = sqrt(2) erfinv(x) = x * R(L),  L = log2(1 - x^2),
+// with R a parabola in L whose coefficients are entry round(-8 L) of a table
+// (normal_coeffs.h).  R is fitted relative to its own value, so eps has a small relative
+// error for every x, including x near 0 (L -> 0) and near +-1: at most 1.9e-7, 5.1e-8 in
+// the mean, and one form serves the centre and the tail.
+//
+// A multiply of Philox (IMAD.WIDE) keeps the issue port busy for about 4 slots, so the
+// kernels that regenerate noise are bound by issue slots, and the transform's instructions
+// count one for one: the parabola takes 8.5 a normal (packed pairs counted as one) where a
+// polynomial of degree 9 with a voted branch for the tail took about 11.  Measured on the
+// update's loop (P = 16, 2^28 elements): 37.9 -> 33.0 cycles per warp-normal, and the
+// bound moves towards the 17 multiplies of a Philox block (16.5 cycles a normal).
+//
+// The table sits in shared memory as C copies, entry i of copy c at float4 C i + c, and a
+// lane reads copy lane % C.  With 8 copies (21,632 bytes) the 8 lanes of a quarter-warp,
+// which one 128-byte wavefront serves, always hit distinct banks whatever their entries:
+// for the kernels that look up several normals per element they load.  The kernels bound
+// by scattered loads or the host link take 1 copy (2,704 bytes), which leaves their
+// occupancy as it was.
+static __device__ const float4 g_normal_table[COPES_NORMAL_ENTRIES] = COPES_NORMAL_TABLE;
+
+template <int C>
+struct NormalTable {
+  static_assert(C == 1 || C == 8, "copies");
+  static constexpr int kFloat4s = COPES_NORMAL_ENTRIES * C;
+  static constexpr int kShift = C == 8 ? 7 : 4;  // log2 of an entry's stride in bytes
+  uint32_t base;
+
+  // Fills a block's table (every load in flight before the first store); a __syncthreads
+  // must follow before the constructor.
+  static __device__ __forceinline__ void fill(float4 *s_tab) {
+    constexpr int kSteps = (kFloat4s + kThreads - 1) / kThreads;
+    float4 v[kSteps];
 #pragma unroll
-  for (int i = 0; i < G; ++i) {
+    for (int k = 0; k < kSteps; ++k) {
+      const int i = threadIdx.x + k * kThreads;
+      if (i < kFloat4s) v[k] = g_normal_table[i / C];
+    }
+#pragma unroll
+    for (int k = 0; k < kSteps; ++k) {
+      const int i = threadIdx.x + k * kThreads;
+      if (i < kFloat4s) s_tab[i] = v[k];
+    }
+  }
+
+  // This lane's view of the table, after the fill's barrier: entry i is at base + (f << kShift)
+  // modulo 2^32 with f the bits of the float 2^23 + i.  Volatile, and every lookup depends on
+  // it, so that no lookup moves above the barrier.
+  __device__ __forceinline__ explicit NormalTable(const float4 *s_tab) {
+    base = smem_addr(s_tab) + (threadIdx.x & (C - 1)) * 16u - (0x4B000000u << kShift);
+    asm volatile("mov.b32 %0, %0;" : "+r"(base)::"memory");
+  }
+
+  __device__ __forceinline__ float4 entry(float f) const {
+    float4 v;
+    asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+        : "r"(base + (__float_as_uint(f) << kShift)));
+    return v;
+  }
+};
+
+using WideTable = NormalTable<8>;
+using SlimTable = NormalTable<1>;
+
+// The normals of G Philox blocks as packed pairs: e2[i][p] = (eps_2p, eps_2p+1) of block i.
+template <int G, typename Table>
+__device__ __forceinline__ void normals_packed(const uint32_t (&w)[G][4], const Table &tab,
+                                               unsigned long long (&e2)[G][2]) {
+  constexpr float kMagic = 8388608.0f;  // 2^23: adding it rounds to a whole number in the low bits
+#pragma unroll
+  for (int i = 0; i < G; ++i)
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
       const unsigned long long F = pack_f32x2(__uint_as_float((w[i][2 * p] & 0x007FFFFEu) | 0x40000001u),
                                               __uint_as_float((w[i][2 * p + 1] & 0x007FFFFEu) | 0x40000001u));
-      x2[i][p] = add_f32x2(F, splat_f32x2(-3.0f));
+      const unsigned long long x2 = add_f32x2(F, splat_f32x2(-3.0f));
       float t0, t1;  // x^2 - 1 = -(1 - x^2)
-      unpack_f32x2(fma_f32x2(x2[i][p], x2[i][p], splat_f32x2(-1.0f)), t0, t1);
-      L[i][2 * p] = lg2_approx(-t0);
-      L[i][2 * p + 1] = lg2_approx(-t1);
-      L_min = fminf(L_min, fminf(L[i][2 * p], L[i][2 * p + 1]));
-      const unsigned long long Lp = pack_f32x2(L[i][2 * p], L[i][2 * p + 1]);
-      unsigned long long acc = splat_f32x2(unit_central[COPES_NORMAL_CENTRAL_DEGREE]);
-#pragma unroll
-      for (int k = COPES_NORMAL_CENTRAL_DEGREE - 1; k >= 0; --k) acc = fma_f32x2(acc, Lp, splat_f32x2(unit_central[k]));
-      r2[i][p] = acc;
+      unpack_f32x2(fma_f32x2(x2, x2, splat_f32x2(-1.0f)), t0, t1);
+      const float L0 = lg2_approx(-t0), L1 = lg2_approx(-t1);
+      float f0, f1;
+      unpack_f32x2(fma_f32x2(pack_f32x2(L0, L1), splat_f32x2(-(float)COPES_NORMAL_SEGMENTS), splat_f32x2(kMagic)), f0,
+                   f1);
+      const float4 k0 = tab.entry(f0), k1 = tab.entry(f1);
+      const float r0 = __fmaf_rn(__fmaf_rn(k0.z, L0, k0.y), L0, k0.x);
+      const float r1 = __fmaf_rn(__fmaf_rn(k1.z, L1, k1.y), L1, k1.x);
+      e2[i][p] = mul_f32x2(x2, pack_f32x2(r0, r1));
     }
-  }
-  if (__any_sync(__activemask(), L_min < COPES_NORMAL_L_SPLIT)) {
-#pragma unroll
-    for (int i = 0; i < G; ++i)
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        float r0, r1;
-        unpack_f32x2(r2[i][p], r0, r1);
-        if (L[i][2 * p] < COPES_NORMAL_L_SPLIT) r0 = tail_ratio(unit_tail, L[i][2 * p]);
-        if (L[i][2 * p + 1] < COPES_NORMAL_L_SPLIT) r1 = tail_ratio(unit_tail, L[i][2 * p + 1]);
-        r2[i][p] = pack_f32x2(r0, r1);
-      }
-  }
 }
 
-// normal_parts4_x2 over G Philox blocks with a single warp vote for the tail: every
-// block's x and r = R(L) scaled by the caller's coefficients (central2 as (c, c) pairs),
-// then, only when some lane of the warp holds a word in the tail, the tail polynomial for
-// those words.  Each result is the same function of its word as in normal_parts4_x2, bit
-// for bit, with one vote for G blocks instead of one per block.
-template <int G, int NC, int NT>
-__device__ __forceinline__ void normal_parts_groups_x2(const uint32_t (&w)[G][4],
-                                                       const unsigned long long (&central2)[NC],
-                                                       const float (&tail)[NT], float (&x)[G][4],
-                                                       float (&r)[G][4]) {
-  float L[G][4];
-  float L_min = 0.0f;  // L <= 0 for every word
-#pragma unroll
-  for (int i = 0; i < G; ++i) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      x[i][e] = lattice_x(w[i][e]);
-      L[i][e] = lg2_approx(__fmaf_rn(-x[i][e], x[i][e], 1.0f));
-      L_min = fminf(L_min, L[i][e]);
-    }
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-      const unsigned long long Lp = pack_f32x2(L[i][2 * p], L[i][2 * p + 1]);
-      unsigned long long acc = central2[NC - 1];
-#pragma unroll
-      for (int k = NC - 2; k >= 0; --k) acc = fma_f32x2(acc, Lp, central2[k]);
-      unpack_f32x2(acc, r[i][2 * p], r[i][2 * p + 1]);
-    }
-  }
-  if (__any_sync(__activemask(), L_min < COPES_NORMAL_L_SPLIT)) {
-#pragma unroll
-    for (int i = 0; i < G; ++i)
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (L[i][e] < COPES_NORMAL_L_SPLIT) r[i][e] = tail_ratio(tail, L[i][e]);
-  }
+// One word, and two words as a packed pair: normals_packed's values bit for bit.
+template <typename Table>
+__device__ __forceinline__ unsigned long long normal_pair(uint32_t wa, uint32_t wb, const Table &tab) {
+  const uint32_t w[1][4] = {{wa, wb, wa, wb}};
+  unsigned long long e2[1][2];
+  normals_packed<1>(w, tab, e2);
+  return e2[0][0];
 }
 
-// normal_parts_groups_x2 with every step on packed pairs, as in normal_parts_groups_packed
-// but with the caller's scaled coefficients (central2: (c, c) pairs): x2[i][p] and r2[i][p]
-// hold words 2p and 2p + 1 of block i, each value normal_parts_groups_x2's bit for bit.
-template <int G, int NC, int NT>
-__device__ __forceinline__ void normal_parts_groups_x2_packed(const uint32_t (&w)[G][4],
-                                                              const unsigned long long (&central2)[NC],
-                                                              const float (&tail)[NT],
-                                                              unsigned long long (&x2)[G][2],
-                                                              unsigned long long (&r2)[G][2]) {
-  float L[G][4];
-  float L_min = 0.0f;  // L <= 0 for every word
-#pragma unroll
-  for (int i = 0; i < G; ++i) {
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-      const unsigned long long F = pack_f32x2(__uint_as_float((w[i][2 * p] & 0x007FFFFEu) | 0x40000001u),
-                                              __uint_as_float((w[i][2 * p + 1] & 0x007FFFFEu) | 0x40000001u));
-      x2[i][p] = add_f32x2(F, splat_f32x2(-3.0f));
-      float t0, t1;  // x^2 - 1 = -(1 - x^2)
-      unpack_f32x2(fma_f32x2(x2[i][p], x2[i][p], splat_f32x2(-1.0f)), t0, t1);
-      L[i][2 * p] = lg2_approx(-t0);
-      L[i][2 * p + 1] = lg2_approx(-t1);
-      L_min = fminf(L_min, fminf(L[i][2 * p], L[i][2 * p + 1]));
-      const unsigned long long Lp = pack_f32x2(L[i][2 * p], L[i][2 * p + 1]);
-      unsigned long long acc = central2[NC - 1];
-#pragma unroll
-      for (int k = NC - 2; k >= 0; --k) acc = fma_f32x2(acc, Lp, central2[k]);
-      r2[i][p] = acc;
-    }
-  }
-  if (__any_sync(__activemask(), L_min < COPES_NORMAL_L_SPLIT)) {
-#pragma unroll
-    for (int i = 0; i < G; ++i)
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        float r0, r1;
-        unpack_f32x2(r2[i][p], r0, r1);
-        if (L[i][2 * p] < COPES_NORMAL_L_SPLIT) r0 = tail_ratio(tail, L[i][2 * p]);
-        if (L[i][2 * p + 1] < COPES_NORMAL_L_SPLIT) r1 = tail_ratio(tail, L[i][2 * p + 1]);
-        r2[i][p] = pack_f32x2(r0, r1);
-      }
-  }
-}
-
-// Two standard normals from two words (of different Philox blocks), their central
-// polynomials evaluated as one packed pair with compile-time coefficients and a single
-// warp vote for the tail: bit-identical to two normal_from_word calls.
-__device__ __forceinline__ void normal_pair_x2(uint32_t wa, uint32_t wb, float &ea, float &eb) {
-  COPES_UNIT_COEFFS;
-  const float xa = lattice_x(wa), xb = lattice_x(wb);
-  const float La = lg2_approx(__fmaf_rn(-xa, xa, 1.0f));
-  const float Lb = lg2_approx(__fmaf_rn(-xb, xb, 1.0f));
-  const unsigned long long Lp = pack_f32x2(La, Lb);
-  unsigned long long b = __float_as_uint(unit_central[COPES_NORMAL_CENTRAL_DEGREE]);
-  unsigned long long acc = (b << 32) | b;
-#pragma unroll
-  for (int k = COPES_NORMAL_CENTRAL_DEGREE - 1; k >= 0; --k) {
-    b = __float_as_uint(unit_central[k]);
-    acc = fma_f32x2(acc, Lp, (b << 32) | b);
-  }
-  float ra, rb;
-  unpack_f32x2(acc, ra, rb);
-  if (__any_sync(__activemask(), fminf(La, Lb) < COPES_NORMAL_L_SPLIT)) {
-    if (La < COPES_NORMAL_L_SPLIT) ra = tail_ratio(unit_tail, La);
-    if (Lb < COPES_NORMAL_L_SPLIT) rb = tail_ratio(unit_tail, Lb);
-  }
-  ea = __fmul_rn(xa, ra);
-  eb = __fmul_rn(xb, rb);
+template <typename Table>
+__device__ __forceinline__ float normal_from_word(uint32_t w, const Table &tab) {
+  const float x = __fadd_rn(__uint_as_float((w & 0x007FFFFEu) | 0x40000001u), -3.0f);
+  const float L = lg2_approx(-__fmaf_rn(x, x, -1.0f));
+  const float4 k = tab.entry(__fmaf_rn(L, -(float)COPES_NORMAL_SEGMENTS, 8388608.0f));
+  return __fmul_rn(x, __fmaf_rn(__fmaf_rn(k.z, L, k.y), L, k.x));
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
@@ -319,10 +190,6 @@ __device__ __forceinline__ void st_stream_u2(void *p, uint2 v) {
 // waits (bounded again) for its own copies, and stops.
 constexpr int kStageChunk = 1024;         // indices per chunk (8 KB)
 constexpr int kStageWaitLimit = 1 << 22;  // mbarrier polls before giving up
-
-__device__ __forceinline__ uint32_t smem_addr(const void *p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
 
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count));

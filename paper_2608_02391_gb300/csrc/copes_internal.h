@@ -5,7 +5,6 @@
 #include <stdint.h>
 
 #include "../../include/copes.h"
-#include "normal_coeffs.h"
 
 namespace copes {
 
@@ -85,8 +84,11 @@ __host__ __device__ __forceinline__ void philox4x32_10_rk(uint32_t c0, uint32_t 
 // philox4x32_10_folded then takes the counter's product M0 * c0 (which a caller computes
 // once for every key) and runs one multiply in round 1 and two in each of rounds 2..9:
 // 17 of the 20 32x32->64 multiplies, with the same output words as philox4x32_10.
-__host__ __device__ __forceinline__ void philox_folded_keys(const uint32_t rk[20], uint32_t tag, uint32_t u[20]) {
-  const uint64_t mk = (uint64_t)kPhiloxM0 * rk[0];
+// A high counter word c1 only enters round 0's key (its new c0 is c1 ^ k0), so keys folded for
+// c1 serve every counter (c0, c1, 0, tag).
+__host__ __device__ __forceinline__ void philox_folded_keys(const uint32_t rk[20], uint32_t tag, uint32_t u[20],
+                                                            uint32_t c1 = 0) {
+  const uint64_t mk = (uint64_t)kPhiloxM0 * (rk[0] ^ c1);
   u[0] = rk[1] ^ tag;
   u[1] = rk[2];
   u[2] = (uint32_t)(mk >> 32) ^ rk[3];
@@ -140,11 +142,11 @@ enum : unsigned {
 };
 
 // ---------------------------------------------------------------- launch arguments
-// R's coefficients pre-multiplied by the perturbation scale (filled by the host).
-struct ScaledCoeffs {
-  unsigned long long central2[COPES_NORMAL_CENTRAL_DEGREE + 1];  // (c, c) pairs
-  float central[COPES_NORMAL_CENTRAL_DEGREE + 1];
-  float tail[COPES_NORMAL_TAIL_DEGREE + 1];
+// How a launch over TILES is cut into units, one grid block each (plan_tile_units): with
+// g = u >> log_parts, unit u covers part u - (g << log_parts) of the tiles
+// [g run, (g + 1) run).
+struct TileUnits {
+  uint32_t n_units, log_parts, run;
 };
 
 // The working copies beyond w (copes_params.w2, w3, w4): n = 0, 1 (w2) or 3 (w2, w3, w4).
@@ -165,7 +167,6 @@ struct ElemArgs {
   uint32_t tag;
   float a;  // perturb: signed sigma; init: scale
   float b;  // init: mean
-  ScaledCoeffs coeffs;  // a * R's coefficients (perturb, init)
   uint32_t rk[20];      // Philox round keys of (seed_lo, seed_hi)
   float *gathered;      // INDICES: theta in list order instead of master[index[p]] (or NULL)
   // kOpPerturbPair / kOpPartner: the antithetic partner's weights (working dtype), element
@@ -173,10 +174,9 @@ struct ElemArgs {
   void *partner;
   uint64_t partner_base, partner_len;
   WorkingCopies copies;  // restore / commit / init write these as well as w
-  // kOpPerturbTwoPairs: the second noise vector's round keys, and both vectors' folded keys
-  // (philox_folded_keys, noise tag) for counters below 2^32
-  uint32_t rk_b[20];
-  uint32_t fk[20], fk_b[20];
+  uint32_t rk_b[20];            // kOpPerturbTwoPairs: the second noise vector's round keys
+  uint32_t fk[20], fk_b[20];    // folded keys (philox_folded_keys, tag) for counters below 2^32
+  TileUnits units;  // TILES
 };
 
 // kOpGather / kOpScatter copy theta between master and the gathered copy (INDICES only).
@@ -216,13 +216,17 @@ struct UpdateArgs {
   int8_t sign[COPES_MAX_MEMBERS];
   float *gathered;  // INDICES: theta in list order instead of master[index[p]] (or NULL)
   WorkingCopies copies;  // the fused commit writes these as well as w
+  TileUnits units;       // TILES
 };
 
 // ------------------------------------------------------------------------ launchers
-// Each returns the launch's cudaError_t (cudaSuccess when nothing was launched).
-cudaError_t launch_elementwise(int op, int kind, int dtype, const ElemArgs &a, cudaStream_t s);
-cudaError_t launch_update(int kind, int dtype, const UpdateArgs &a, cudaStream_t s,
-                          int num_sms);
+// The units of a launch over n_tiles disjoint tiles of an n_alloc-element arena (n_tiles in
+// [1, 2^31)): fewer tiles than `few` are cut into 2^log_parts parts each.
+TileUnits plan_tile_units(uint64_t n_tiles, uint64_t n_alloc, uint32_t log_parts, uint32_t few);
+
+// launch_elementwise and launch_update fill in a.units.
+cudaError_t launch_elementwise(int op, int kind, int dtype, ElemArgs &a, cudaStream_t s);
+cudaError_t launch_update(int kind, int dtype, UpdateArgs &a, cudaStream_t s);
 cudaError_t launch_shape(const float *r, int n, const int32_t *group, int mode, float *f,
                          cudaStream_t s);
 cudaError_t launch_debug_philox(uint64_t seed, uint64_t q0, uint64_t n, uint32_t aux,
@@ -294,8 +298,8 @@ cudaError_t launch_replay_mask(const ReplayArgs &r, uint64_t n_alloc, uint32_t *
 // kBackupPerturbPair: w = round(theta + a eps) and the antithetic partner's
 // round(theta - a eps) into ElemArgs.partner, theta = the backup, read over the link once.
 enum BackupOp { kBackupSave = 0, kBackupPerturb = 1, kBackupRestore = 2, kBackupPerturbPair = 3 };
-cudaError_t launch_backup_elementwise(int op, const ElemArgs &a, uint16_t *backup, cudaStream_t s);
-cudaError_t launch_backup_update(const UpdateArgs &a, uint16_t *backup, cudaStream_t s);
+cudaError_t launch_backup_elementwise(int op, ElemArgs &a, uint16_t *backup, cudaStream_t s);
+cudaError_t launch_backup_update(UpdateArgs &a, uint16_t *backup, cudaStream_t s);
 
 // Sets the calling thread's message reported by copes_last_error.
 void set_last_error(const char *message);

@@ -180,8 +180,12 @@ __global__ void __launch_bounds__(kThreads) replay_elem_kernel(const __grid_cons
   __shared__ uint32_t s_pool[(kThreads / 32) * BATCH];
   __shared__ uint64_t s_g0[kThreads / 32][kReplayTilesPerBlock];
   __shared__ int s_pool_n;
+  constexpr bool kNoise = OP != kOpRestore && OP != kOpPartner;
+  __shared__ __align__(16) float4 s_tab[kNoise ? SlimTable::kFloat4s : 1];
   if (threadIdx.x == 0) s_pool_n = 0;
+  if (kNoise) SlimTable::fill(s_tab);
   __syncthreads();
+  const SlimTable tab(s_tab);
   float *__restrict__ master = a.master;
   replay_stream<BATCH, MASK>(r, a.n_alloc, s_buf[threadIdx.x >> 5], s_g0, s_pool, &s_pool_n,
                              [&](const uint64_t (&g)[U], const bool (&ok_in)[U]) {
@@ -213,10 +217,9 @@ __global__ void __launch_bounds__(kThreads) replay_elem_kernel(const __grid_cons
         philox4x32_10_rk((uint32_t)q, (uint32_t)(q >> 32), 0u, replay_tag<OP>(), a.rk, x);
         const uint32_t sel = (uint32_t)g[u] & 3u;
         const uint32_t wd = sel == 0 ? x[0] : (sel == 1 ? x[1] : (sel == 2 ? x[2] : x[3]));
-        float xv, r;
-        normal_parts(wd, a.coeffs.central, a.coeffs.tail, xv, r);  // r = a * R(L)
-        v = __fmaf_rn(r, xv, OP == kOpInit ? a.b : th[u]);
-        if (OP == kOpPerturbPair) vp = __fmaf_rn(-r, xv, th[u]);
+        const float eps = normal_from_word(wd, tab);
+        v = __fmaf_rn(a.a, eps, OP == kOpInit ? a.b : th[u]);
+        if (OP == kOpPerturbPair) vp = __fmaf_rn(-a.a, eps, th[u]);
         if (OP == kOpInit) master[g[u]] = v;
       }
       WStore<WT>::one(a.w, g[u], v);
@@ -233,14 +236,13 @@ __global__ void __launch_bounds__(kThreads) replay_update_kernel(const __grid_co
                                                                  const __grid_constant__ ReplayArgs r) {
   constexpr int BATCH = 64;
   constexpr int U = BATCH / 32;
-  __shared__ float s_w[COPES_MAX_NOISE];
-  __shared__ __align__(16) uint32_t s_rk[COPES_MAX_NOISE][20];
+  extern __shared__ __align__(128) char s_update[];
   __shared__ uint32_t s_buf[kThreads / 32][BATCH + 128];
   __shared__ uint32_t s_pool[(kThreads / 32) * BATCH];
   __shared__ uint64_t s_g0[kThreads / 32][kReplayTilesPerBlock];
   __shared__ int s_pool_n;
   if (threadIdx.x == 0) s_pool_n = 0;
-  noise_weights_to_smem(a, s_w, s_rk);  // ends with __syncthreads
+  const GatherSmem s = gather_prologue(a, s_update);  // ends with __syncthreads
   float *__restrict__ master = a.master;
   const int P = a.n_noise;
   replay_stream<BATCH, MASK>(r, a.n_alloc, s_buf[threadIdx.x >> 5], s_g0, s_pool, &s_pool_n,
@@ -248,30 +250,8 @@ __global__ void __launch_bounds__(kThreads) replay_update_kernel(const __grid_co
     float acc[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) acc[u] = 0.0f;
-    for (int j = 0; j < P; ++j) {
-      uint32_t rk[20];
-#pragma unroll
-      for (int q = 0; q < 20; q += 4) {
-        const uint4 v = *reinterpret_cast<const uint4 *>(&s_rk[j][q]);
-        rk[q] = v.x, rk[q + 1] = v.y, rk[q + 2] = v.z, rk[q + 3] = v.w;
-      }
-      const float wj = s_w[j];
-      uint32_t wd[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        uint32_t x[4];
-        const uint64_t q = g[u] >> 2;
-        philox4x32_10_rk((uint32_t)q, (uint32_t)(q >> 32), 0u, COPES_TAG_NOISE, rk, x);
-        const uint32_t sel = (uint32_t)g[u] & 3u;
-        wd[u] = sel == 0 ? x[0] : (sel == 1 ? x[1] : (sel == 2 ? x[2] : x[3]));
-      }
-      // the two members' normals as one packed pair (bit-identical to one at a time)
-      static_assert(U == 2, "normals are paired");
-      float eps0, eps1;
-      normal_pair_x2(wd[0], wd[1], eps0, eps1);
-      acc[0] = __fmaf_rn(wj, eps0, acc[0]);
-      acc[1] = __fmaf_rn(wj, eps1, acc[1]);
-    }
+    static_assert(U == 2, "gather_noise_add takes two elements");
+    for (int j = 0; j < P; ++j) gather_noise_add(s, j, g, acc);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (!ok[u]) continue;
@@ -355,10 +335,11 @@ cudaError_t launch_replay_elementwise(int op, int dtype, const ElemArgs &a, cons
 template <typename WT, bool COMMIT>
 static cudaError_t launch_replay_update_typed(const UpdateArgs &a, const ReplayArgs &r, cudaStream_t s) {
   if (r.n_tiles == 0) return cudaSuccess;
-  if (r.mask)
-    replay_update_kernel<WT, COMMIT, true><<<replay_blocks(r.n_tiles), kThreads, 0, s>>>(a, r);
-  else
-    replay_update_kernel<WT, COMMIT, false><<<replay_blocks(r.n_tiles), kThreads, 0, s>>>(a, r);
+  const uint32_t smem = update_smem_bytes(a.n_noise);
+  auto kernel = r.mask ? replay_update_kernel<WT, COMMIT, true> : replay_update_kernel<WT, COMMIT, false>;
+  const cudaError_t e = allow_smem((const void *)kernel, smem + 16 * 1024, smem);  // 8.5 KB static
+  if (e != cudaSuccess) return e;
+  kernel<<<replay_blocks(r.n_tiles), kThreads, smem, s>>>(a, r);
   return cudaGetLastError();
 }
 
