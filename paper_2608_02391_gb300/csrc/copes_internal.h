@@ -84,13 +84,14 @@ __host__ __device__ __forceinline__ void philox4x32_10_rk(uint32_t c0, uint32_t 
 // philox4x32_10_folded then takes the counter's product M0 * c0 (which a caller computes
 // once for every key) and runs one multiply in round 1 and two in each of rounds 2..9:
 // 17 of the 20 32x32->64 multiplies, with the same output words as philox4x32_10.
-// A high counter word c1 only enters round 0's key (its new c0 is c1 ^ k0), so keys folded for
-// c1 serve every counter (c0, c1, 0, tag).
+// Other words c1 and c2 only enter round 0's result (its new c0 is hi(M1 c2) ^ c1 ^ k0, its new
+// c1 is lo(M1 c2)), so keys folded for them serve every counter (c0, c1, c2, tag).
 __host__ __device__ __forceinline__ void philox_folded_keys(const uint32_t rk[20], uint32_t tag, uint32_t u[20],
-                                                            uint32_t c1 = 0) {
-  const uint64_t mk = (uint64_t)kPhiloxM0 * (rk[0] ^ c1);
+                                                            uint32_t c1 = 0, uint32_t c2 = 0) {
+  const uint64_t m2 = (uint64_t)kPhiloxM1 * c2;
+  const uint64_t mk = (uint64_t)kPhiloxM0 * (rk[0] ^ c1 ^ (uint32_t)(m2 >> 32));
   u[0] = rk[1] ^ tag;
-  u[1] = rk[2];
+  u[1] = rk[2] ^ (uint32_t)m2;
   u[2] = (uint32_t)(mk >> 32) ^ rk[3];
   u[3] = (uint32_t)mk ^ rk[5];
   u[4] = rk[4];
@@ -220,6 +221,13 @@ struct UpdateArgs {
 };
 
 // ------------------------------------------------------------------------ launchers
+// Lets `kernel` take `dynamic` bytes of dynamic shared memory when that and its static share
+// pass the default limit of 48 KB a block (host).
+inline cudaError_t allow_smem(const void *kernel, uint32_t total, uint32_t dynamic) {
+  if (total <= 48u * 1024u) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic);
+}
+
 // The units of a launch over n_tiles disjoint tiles of an n_alloc-element arena (n_tiles in
 // [1, 2^31)): fewer tiles than `few` are cut into 2^log_parts parts each.
 TileUnits plan_tile_units(uint64_t n_tiles, uint64_t n_alloc, uint32_t log_parts, uint32_t few);

@@ -368,11 +368,4 @@ __device__ __forceinline__ void gather_noise_add(const GatherSmem &s, int j, con
   acc[1] = __fmaf_rn(wj, e1, acc[1]);
 }
 
-// Lets `kernel` take `dynamic` bytes of dynamic shared memory when that and its static share
-// pass the default limit of 48 KB a block (host).
-inline cudaError_t allow_smem(const void *kernel, uint32_t total, uint32_t dynamic) {
-  if (total <= 48u * 1024u) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic);
-}
-
 }  // namespace copes
