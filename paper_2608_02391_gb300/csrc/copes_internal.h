@@ -9,7 +9,7 @@
 namespace copes {
 
 constexpr int kThreads = 256;       // threads per block of the elementwise kernels
-constexpr int kIndexSegment = 8192; // indices per block in the gather kernels
+constexpr int kIndexSegment = 8192; // indices per block in the gather kernels, at most
 
 // Philox4x32-10 constants (SC'11, Sec. 3): round multipliers and key (Weyl) increments.
 constexpr uint32_t kPhiloxM0 = 0xD2511F53u;
@@ -133,6 +133,54 @@ __host__ __device__ __forceinline__ void philox4x32_10_folded(uint32_t m0_lo, ui
   out[3] = c3;
 }
 
+// One word of a block: word 2h + odd of the counter whose product M0 c0 is given, with the last
+// two rounds cut to what that word takes.  With the state after round 7, round 9's product for
+// words 0 and 1 is M1 n2, n2 = hi(M0 c0) ^ c3 ^ rk17, and word 0 also takes the low half of
+// round 8's other product, lo(M1 c2); for words 2 and 3 the same with the halves' roles
+// exchanged.  15 wide multiplies and one low one are left of the folded form's 17.
+// Keys (philox_word_keys): row[0 .. 14] as folded; (rk17, rk18) in row[16, 17] for h = 0 and
+// (rk16, rk19) in row[18, 19] for h = 1, the last two rounds' keys; row[15] is free.
+__host__ __device__ __forceinline__ void philox_word_keys(const uint32_t rk[20], uint32_t tag, uint32_t row[20]) {
+  philox_folded_keys(rk, tag, row);
+  row[15] = 0;
+  row[16] = rk[17];
+  row[17] = rk[18];
+  row[18] = rk[16];
+  row[19] = rk[19];
+}
+
+template <typename U>
+__host__ __device__ __forceinline__ uint32_t philox4x32_10_word(uint32_t m0_lo, uint32_t m0_hi, const U &u, bool h,
+                                                                bool odd, uint32_t k8, uint32_t k9) {
+  uint32_t c2 = m0_hi ^ u[0];  // rounds 0 .. 2 as in philox4x32_10_folded
+  uint64_t p1 = (uint64_t)kPhiloxM1 * c2;
+  uint32_t c0 = (uint32_t)(p1 >> 32) ^ u[1];
+  uint32_t c1 = (uint32_t)p1;
+  c2 = u[2] ^ m0_lo;
+  uint64_t p0 = (uint64_t)kPhiloxM0 * c0;
+  p1 = (uint64_t)kPhiloxM1 * c2;
+  c0 = (uint32_t)(p1 >> 32) ^ c1 ^ u[4];
+  c2 = (uint32_t)(p0 >> 32) ^ u[3];
+  c1 = (uint32_t)p1;
+  uint32_t c3 = (uint32_t)p0;
+#pragma unroll
+  for (int r = 3; r < 8; ++r) {
+    p0 = (uint64_t)kPhiloxM0 * c0;
+    p1 = (uint64_t)kPhiloxM1 * c2;
+    const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c1 ^ u[5 + 2 * (r - 3)];
+    const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c3 ^ u[6 + 2 * (r - 3)];
+    c1 = (uint32_t)p1;
+    c3 = (uint32_t)p0;
+    c0 = n0;
+    c2 = n2;
+  }
+  const uint32_t ma = h ? kPhiloxM1 : kPhiloxM0, mb = h ? kPhiloxM0 : kPhiloxM1;
+  const uint32_t ca = h ? c2 : c0, cb = h ? c0 : c2, cx = h ? c1 : c3;
+  const uint32_t n = (uint32_t)((uint64_t)ma * ca >> 32) ^ cx ^ k8;
+  const uint64_t p = (uint64_t)mb * n;
+  return odd ? (uint32_t)p : (uint32_t)(p >> 32) ^ (mb * cb) ^ k9;
+}
+
 // Device error bits (set with atomicOr by a kernel that skipped an access).
 enum : unsigned {
   kErrTileRange = 1u,   // a tile outside [0, n_alloc) or longer than COPES_TILE_MAX
@@ -177,7 +225,8 @@ struct ElemArgs {
   WorkingCopies copies;  // restore / commit / init write these as well as w
   uint32_t rk_b[20];            // kOpPerturbTwoPairs: the second noise vector's round keys
   uint32_t fk[20], fk_b[20];    // folded keys (philox_folded_keys, tag) for counters below 2^32
-  TileUnits units;  // TILES
+  TileUnits units;   // TILES
+  uint32_t segment;  // INDICES: list entries per block
 };
 
 // kOpGather / kOpScatter copy theta between master and the gathered copy (INDICES only).
@@ -218,6 +267,7 @@ struct UpdateArgs {
   float *gathered;  // INDICES: theta in list order instead of master[index[p]] (or NULL)
   WorkingCopies copies;  // the fused commit writes these as well as w
   TileUnits units;       // TILES
+  uint32_t segment;      // INDICES: list entries per block
 };
 
 // ------------------------------------------------------------------------ launchers
@@ -232,7 +282,7 @@ inline cudaError_t allow_smem(const void *kernel, uint32_t total, uint32_t dynam
 // [1, 2^31)): fewer tiles than `few` are cut into 2^log_parts parts each.
 TileUnits plan_tile_units(uint64_t n_tiles, uint64_t n_alloc, uint32_t log_parts, uint32_t few);
 
-// launch_elementwise and launch_update fill in a.units.
+// launch_elementwise and launch_update fill in a.units and a.segment.
 cudaError_t launch_elementwise(int op, int kind, int dtype, ElemArgs &a, cudaStream_t s);
 cudaError_t launch_update(int kind, int dtype, UpdateArgs &a, cudaStream_t s);
 cudaError_t launch_shape(const float *r, int n, const int32_t *group, int mode, float *f,

@@ -244,14 +244,10 @@ __global__ void __launch_bounds__(kThreads) replay_update_kernel(const __grid_co
   if (threadIdx.x == 0) s_pool_n = 0;
   const GatherSmem s = gather_prologue(a, s_update);  // ends with __syncthreads
   float *__restrict__ master = a.master;
-  const int P = a.n_noise;
   replay_stream<BATCH, MASK>(r, a.n_alloc, s_buf[threadIdx.x >> 5], s_g0, s_pool, &s_pool_n,
                              [&](const uint64_t (&g)[U], const bool (&ok)[U]) {
     float acc[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) acc[u] = 0.0f;
-    static_assert(U == 2, "gather_noise_add takes two elements");
-    for (int j = 0; j < P; ++j) gather_noise_add(s, j, g, acc);
+    gather_noise_sum(a, s, g, acc);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (!ok[u]) continue;
@@ -335,7 +331,7 @@ cudaError_t launch_replay_elementwise(int op, int dtype, const ElemArgs &a, cons
 template <typename WT, bool COMMIT>
 static cudaError_t launch_replay_update_typed(const UpdateArgs &a, const ReplayArgs &r, cudaStream_t s) {
   if (r.n_tiles == 0) return cudaSuccess;
-  const uint32_t smem = update_smem_bytes(a.n_noise);
+  const uint32_t smem = gather_smem_bytes(a.n_noise);
   auto kernel = r.mask ? replay_update_kernel<WT, COMMIT, true> : replay_update_kernel<WT, COMMIT, false>;
   const cudaError_t e = allow_smem((const void *)kernel, smem + 16 * 1024, smem);  // 8.5 KB static
   if (e != cudaSuccess) return e;

@@ -30,3 +30,22 @@ def test_folded_keys_for_any_counter_match_the_oracle(tmp_path):
     for (k, c0, c1, c2, tag), line in zip(cases, out):
         ref = oracle.philox4x32_10([c0, c1, c2, tag], [k & 0xFFFFFFFF, k >> 32])
         assert [int(v) for v in line.split()] == [int(v) for v in ref], (k, c0, c1, c2, tag)
+
+
+def test_single_words_match_the_oracle(tmp_path):
+    import oracle
+    cxx, inc = shutil.which("g++"), _cuda_include()
+    if not cxx or not inc:
+        pytest.skip("g++ or the CUDA headers are not available")
+    exe = str(tmp_path / "philox_word")
+    subprocess.run([cxx, "-std=c++17", "-O1", "-I", inc, os.path.join(ROOT, "tests", "philox_word_main.cpp"),
+                    "-o", exe], check=True, capture_output=True, text=True)
+    rng = np.random.default_rng(5)
+    cases = [(k, c) for k in [0, 33, 2**64 - 1] + [int(v) for v in rng.integers(0, 2**63, 20)]
+             for c in [0, 1, 2**31, 2**32 - 1] + [int(v) for v in rng.integers(0, 2**32, 20)]]
+    out = subprocess.run([exe], input="".join("%d %d\n" % c for c in cases), capture_output=True, text=True,
+                         check=True).stdout.splitlines()
+    assert len(out) == len(cases)
+    for (k, c), line in zip(cases, out):
+        ref = oracle.philox4x32_10([c, 0, 0, 0], [k & 0xFFFFFFFF, k >> 32])
+        assert [int(v) for v in line.split()] == [int(v) for v in ref], (k, c)
