@@ -115,30 +115,31 @@ def perturb_members(arena: copes.Arena, sub: copes.SubspaceHandle, members: Sequ
         perturb, pair, copy = copes.backup_perturb, copes.backup_perturb_pair, copes.backup_perturb_partner
     else:
         perturb, pair, copy = copes.perturb, copes.perturb_pair, copes.perturb_partner
+    nid, sign, seeds = np.asarray(nid).tolist(), np.asarray(sign).tolist(), [int(x) for x in seeds]
+    two_pairs = partner is not None and partner.two_pairs and sub.kind == copes.SUBSPACE_TILES
     staged = None  # the member whose weights the partner buffer holds
     ready = {}     # member -> the working copy that already holds its weights
     for pos, i in enumerate(members):
-        nxt = members[pos + 1] if pos + 1 < len(members) else None
-        seed, ss = int(seeds[nid[i]]), float(sign[i]) * s_k
         where = None if arena is None else arena.w
-        quad = (members[pos:pos + 4] if partner is not None and partner.two_pairs
-                and sub.kind == copes.SUBSPACE_TILES else [])
         if i in ready:
             where = ready.pop(i)
         elif staged == i and partner.in_place:
             where = partner.buf
         elif staged == i:
-            _timed(events, "partner", lambda: copy(arena, sub, partner.buf, partner.base))
-        elif (len(quad) == 4 and _antithetic(nid, sign, quad[0], quad[1]) and _antithetic(nid, sign, quad[2], quad[3])
-              and sign[quad[2]] == sign[i]):
-            seed_b = int(seeds[nid[quad[2]]])
-            _timed(events, "perturb", lambda: copes.perturb_two_pairs(arena, sub, seed, seed_b, ss))
-            ready = {quad[1]: arena.w2, quad[2]: arena.w3, quad[3]: arena.w4}
-        elif partner is not None and nxt is not None and _antithetic(nid, sign, i, nxt):
-            _timed(events, "perturb", lambda: pair(arena, sub, seed, ss, partner.buf, partner.base))
-            staged = nxt
+            _timed(events, "partner", copy, arena, sub, partner.buf, partner.base)
         else:
-            _timed(events, "perturb", lambda: perturb(arena, sub, seed, ss))
+            seed, ss = seeds[nid[i]], float(sign[i]) * s_k
+            nxt = members[pos + 1] if partner is not None and pos + 1 < len(members) else None
+            quad = members[pos:pos + 4] if two_pairs else ()
+            if (len(quad) == 4 and _antithetic(nid, sign, quad[0], quad[1]) and _antithetic(nid, sign, quad[2], quad[3])
+                    and sign[quad[2]] == sign[i]):
+                _timed(events, "perturb", copes.perturb_two_pairs, arena, sub, seed, seeds[nid[quad[2]]], ss)
+                ready = {quad[1]: arena.w2, quad[2]: arena.w3, quad[3]: arena.w4}
+            elif nxt is not None and _antithetic(nid, sign, i, nxt):
+                _timed(events, "perturb", pair, arena, sub, seed, ss, partner.buf, partner.base)
+                staged = nxt
+            else:
+                _timed(events, "perturb", perturb, arena, sub, seed, ss)
         if arena is not None:
             arena.live = where
         live(i)
@@ -233,13 +234,13 @@ def sync_step(arena: copes.Arena, subs: Sequence[copes.SubspaceHandle], iteratio
     return f
 
 
-def _timed(events: Optional[dict], name: str, fn):
+def _timed(events: Optional[dict], name: str, fn, *args):
     if events is None:
-        return fn()
+        return fn(*args)
     start = torch.cuda.Event(enable_timing=True)
     end = torch.cuda.Event(enable_timing=True)
     start.record()
-    out = fn()
+    out = fn(*args)
     end.record()
     events.setdefault(name, []).append((start, end))
     return out
