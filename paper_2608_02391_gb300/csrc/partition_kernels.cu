@@ -154,7 +154,7 @@ struct ListTable {
 // warps.  So a group of 4 elements is hashed once and the lists are written in full lines.
 // 494M elements, K = 16: 4.04 ms when every element hashed its own group and went to its list
 // directly, 2.79 ms with ranks from warp matches instead of private columns.
-constexpr int kScatterGroups = (int)kHashTile / 4 / kPartThreads;  // consecutive groups a thread
+constexpr uint32_t kScatterGroups = (uint32_t)kHashTile / 4 / kPartThreads;  // consecutive groups a thread
 constexpr uint32_t kScatterSmem(int K) { return (uint32_t)kHashTile * 2 + (uint32_t)K * kPartThreads * 4; }
 
 __global__ void __launch_bounds__(kPartThreads) hash_scatter_kernel(
@@ -172,16 +172,17 @@ __global__ void __launch_bounds__(kPartThreads) hash_scatter_kernel(
   const Bucket bucket(K);
   const uint32_t g0 = threadIdx.x * kScatterGroups;  // the thread's first group
   uint32_t packed[kScatterGroups];                   // its groups' buckets
+  const uint32_t mine = min(t.len - min(t.len, g0 * 4), kScatterGroups * 4u);  // its elements
 #pragma unroll
-  for (int i = 0; i < kScatterGroups; ++i) {
+  for (uint32_t i = 0; i < kScatterGroups; ++i) {
     uint32_t x[4];
     t.words(g0 + i, x);
     packed[i] = 0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (uint32_t j = 0; j < 4; ++j) {
       const uint32_t b = bucket(x[j]);
       packed[i] |= b << (8 * j);
-      if ((g0 + i) * 4 + j < t.len) atomicAdd(column + b * kPartThreads, 1u);
+      if (i * 4 + j < mine) atomicAdd(column + b * kPartThreads, 1u);
     }
   }
   __syncthreads();
@@ -213,27 +214,23 @@ __global__ void __launch_bounds__(kPartThreads) hash_scatter_kernel(
   }
   __syncthreads();
 #pragma unroll
-  for (int i = 0; i < kScatterGroups; ++i)
+  for (uint32_t i = 0; i < kScatterGroups; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const uint32_t e = (g0 + i) * 4 + j;
-      if (e < t.len) s_sorted[atomicAdd(column + (packed[i] >> (8 * j) & 0xFFu) * kPartThreads, 1u)] = (uint16_t)e;
+      if (i * 4 + j < mine)
+        s_sorted[atomicAdd(column + (packed[i] >> (8 * j) & 0xFFu) * kPartThreads, 1u)] = (uint16_t)((g0 + i) * 4 + j);
     }
   __syncthreads();
-  // the buckets' stretches in pieces of 256, dealt to the warps in turn
+  // the buckets' stretches: whole ones dealt to the warps, or all of them to all warps when
+  // they are fewer
   const int64_t first = (int64_t)(t.T.offset + t.e0);
-  uint32_t turn = 0;
-  for (int k = 0; k < K; ++k) {
+  const bool whole = K >= kWarps;
+  const uint32_t lane0 = whole ? 0u : warp * 32u, stride = whole ? 32u : kPartThreads;
+  for (int k = whole ? warp : 0; k < K; k += whole ? kWarps : 1) {
     const uint32_t b = s_start[k], n = s_start[k + 1] - b;
-    if (n == 0) continue;
     long long *list = reinterpret_cast<long long *>(lists.list[k] + offsets[tile * K + k]);
-    for (uint32_t c = (warp - turn) % kWarps * 256u; c < n; c += kWarps * 256u) {
-      const uint32_t left = min(n - c, 256u);
-#pragma unroll
-      for (uint32_t i = 0; i < 256; i += 32)
-        if (i + lane < left) __stcs(list + c + i + lane, (long long)(first + s_sorted[b + c + i + lane]));
-    }
-    turn = (turn + (n + 255) / 256) % kWarps;
+#pragma unroll 4
+    for (uint32_t i = lane0 + lane; i < n; i += stride) __stcs(list + i, (long long)(first + s_sorted[b + i]));
   }
 }
 
