@@ -175,6 +175,12 @@ __device__ __forceinline__ uint16_t to_bf16_bits(float x) {
 __device__ __forceinline__ float4 ld_stream_f4(const float *p) {
   return __ldcs(reinterpret_cast<const float4 *>(p));
 }
+// 32 bytes (aligned to as many) in one load, past the L1.
+__device__ __forceinline__ void ld_stream_f8(const float *p, float (&x)[4], float (&y)[4]) {
+  asm volatile("ld.global.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(y[0]), "=f"(y[1]), "=f"(y[2]), "=f"(y[3])
+               : "l"(p));
+}
 __device__ __forceinline__ void st_stream_f4(float *p, float4 v) {
   __stcs(reinterpret_cast<float4 *>(p), v);
 }

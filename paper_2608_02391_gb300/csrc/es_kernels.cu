@@ -130,6 +130,57 @@ __device__ __forceinline__ void elem_step(const ElemArgs &a, const WideTable &ta
   }
 }
 
+// The two pairs' bf16 step by octets: G / 2 runs of two adjacent groups a thread, at
+// b + off + 8 kThreads i, each with one 32-byte load and one 16-byte store a value where
+// elem_step has two of half the size: fewer memory instructions in a launch bound by its issue
+// slots.  2^28 elements take 510 us instead of 523 (518 with a product M0 q for each group,
+// where the second is the first's plus M0).  The pair and the perturb (320 -> 311 and 258 -> 257
+// us, but 8.01 -> 8.08 and 7.4 -> 8.4 of 4M elements) keep elem_step, as do elem_part's units
+// (10.1 -> 11.0 us of 3M elements with octets).
+template <int G>
+__device__ __forceinline__ void two_pairs_octets(const ElemArgs &a, const WideTable &tab, uint64_t b, uint32_t off) {
+  constexpr int OP = kOpPerturbTwoPairs, H = G / 2;
+  const float *__restrict__ mt = a.master + b;
+  float th[G][4];
+#pragma unroll
+  for (int i = 0; i < H; ++i) ld_stream_f8(mt + off + 8u * kThreads * i, th[2 * i], th[2 * i + 1]);
+  uint32_t w[2 * G][4];
+  const uint32_t q0 = (uint32_t)(b >> 2);
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    uint64_t m = (uint64_t)kPhiloxM0 * (q0 + ((off >> 2) + 2 * kThreads * i));
+#pragma unroll
+    for (int h = 0; h < 2; ++h, m += kPhiloxM0) {
+      philox4x32_10_folded((uint32_t)m, (uint32_t)(m >> 32), a.fk, w[4 * i + 2 * h]);
+      philox4x32_10_folded((uint32_t)m, (uint32_t)(m >> 32), a.fk_b, w[4 * i + 2 * h + 1]);
+    }
+  }
+  unsigned long long e2[2 * G][2];
+  normals_packed<2 * G>(w, tab, e2);
+#pragma unroll
+  for (int i = 0; i < H; ++i) {
+    const uint64_t g = b + off + 8u * kThreads * i;
+    float v[2][4][4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) group_values<OP>(a, &e2[2 * (2 * i + h)], th[2 * i + h], v[h]);
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+      __stcs(reinterpret_cast<uint4 *>(reinterpret_cast<uint16_t *>(m == 0 ? a.w : a.copies.p[m - 1]) + g),
+             make_uint4(pack_bf16x2(v[0][m][0], v[0][m][1]), pack_bf16x2(v[0][m][2], v[0][m][3]),
+                        pack_bf16x2(v[1][m][0], v[1][m][1]), pack_bf16x2(v[1][m][2], v[1][m][3])));
+  }
+}
+
+// Whether an octet at b starts on 32 bytes of theta and 16 of each buffer.  (The addresses
+// themselves: the same answer from b and the bases, 524 us for 512 of 2^28 elements, is
+// compiled to a slower loop.)
+__device__ __forceinline__ bool octets_aligned(const ElemArgs &a, uint64_t b) {
+  uintptr_t w = reinterpret_cast<uintptr_t>(reinterpret_cast<uint16_t *>(a.w) + b);
+#pragma unroll
+  for (int m = 0; m < 3; ++m) w |= reinterpret_cast<uintptr_t>(reinterpret_cast<uint16_t *>(a.copies.p[m]) + b);
+  return ((reinterpret_cast<uintptr_t>(a.master + b) | w << 1 | b * 4) & 31) == 0;
+}
+
 // The default tile, with every bound a compile-time constant (a runtime bound spilled
 // registers and cost the two-pairs perturb 5%).
 constexpr uint32_t kElemSpan = 16384;
@@ -138,6 +189,15 @@ template <int OP, typename WT, int G>
 __device__ __forceinline__ void elem_span(const ElemArgs &a, const WideTable &tab, uint64_t b, NextUnit &next) {
   constexpr uint32_t kStep = 4u * kThreads * G;
   static_assert(kElemSpan % kStep == 0, "a span is whole steps");
+  if constexpr (OP == kOpPerturbTwoPairs && sizeof(WT) == 2) {
+    if (octets_aligned(a, b)) {
+      for (uint32_t at = 0; at < kElemSpan; at += kStep) {
+        if (at == kElemSpan - kStep) next.ask();
+        two_pairs_octets<G>(a, tab, b, at + 8u * threadIdx.x);
+      }
+      return;
+    }
+  }
   for (uint32_t at = 0; at < kElemSpan; at += kStep) {
     if (at == kElemSpan - kStep) next.ask();
     elem_step<OP, WT, G, true>(a, tab, b, at + 4u * threadIdx.x);

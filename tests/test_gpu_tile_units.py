@@ -101,3 +101,21 @@ def test_invalid_tile_in_a_run_is_left_out(copes):
     for t in bad:
         want[t * tile:(t + 1) * tile] = 0
     assert torch.equal(a.w, want)
+
+
+@pytest.mark.parametrize("offset", [0, 4])  # floats before theta: 32-byte aligned or not
+@pytest.mark.parametrize("begin", [0, 4, 8, 3])
+def test_two_pairs_over_whole_tiles_equal_pairs(copes, begin, offset):
+    """Enough default tiles to stay whole: by octets where theta's addresses allow them."""
+    n = begin + 1300 * 16_384 + 5
+    master = (torch.randn(n + offset, device="cuda") * 0.02)[offset:]
+    a = copes.Arena(torch.zeros(n, dtype=torch.bfloat16, device="cuda"), master,
+                    *[torch.zeros(n, dtype=torch.bfloat16, device="cuda") for _ in range(3)])
+    sub = copes.tiles_from_ranges([(begin, n)], tile_size=16_384)
+    copes.perturb_two_pairs(a, sub, *SEEDS, 1e-3)
+    got = [c.clone() for c in a.copies]
+    for k, seed in enumerate(SEEDS):
+        a.w.zero_(), a.w2.zero_()
+        copes.perturb_pair(a, sub, seed, 1e-3, a.w2)
+        assert torch.equal(a.w, got[2 * k]) and torch.equal(a.w2, got[2 * k + 1])
+    copes.check()
