@@ -27,6 +27,13 @@ using copes::UpdateArgs;
 // 39.2 / 36.5 / 36.3 us; the update (P = 16) of 2^18, 2^20 and 4M elements 47.8 / 46.0 /
 // 9.3, 47.9 / 46.2 / 21.5 and 85.3 / 79.8 / 62.9 us, of 14.9M elements 234 / 215 / 221 us;
 // tiles of 1,000 elements joined, 11.1M elements: perturb 29.0 -> 18.8 us, update 351 -> 178.
+// The bound is loose by as much as the subspace is a part of the arena, and a run then holds
+// less than it says: short tiles are joined while 500 units are left, and those of a middling
+// bound up to 32,768 elements by it while there are eight waves of units.  Tiles of 1,000 in a
+// third of the arena, 4, 11.1 and 134M elements, only eight waves of at most 16,384 / these:
+// perturb 17.0 / 10.4, 30.6 / 20.7 and 205 / 172 us, update (P = 7) 38.2 / 36.2, 92.9 / 86.4 and
+// 919 / 881.  From 3,500 on whole tiles are long enough (aligned tiles of 4,096, 11.1M
+// elements: pair 17.2 / 19.8).
 copes::TileUnits copes::plan_tile_units(uint64_t n_tiles, uint64_t n_alloc, uint32_t log_parts, uint32_t few) {
   TileUnits u{(uint32_t)n_tiles, 0, 1};
   const uint64_t bound = std::max<uint64_t>(1, n_alloc / n_tiles);  // >= the mean tile length
@@ -35,8 +42,10 @@ copes::TileUnits copes::plan_tile_units(uint64_t n_tiles, uint64_t n_alloc, uint
   } else if (n_tiles < 500) {
     while ((n_tiles << (u.log_parts + 1)) <= 500 && (bound >> (u.log_parts + 1)) >= 1024) ++u.log_parts;
   } else {
-    const uint64_t left = bound < 2048 ? 500 : 8 * 608;
-    u.run = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>({32, 16384 / bound, n_tiles / left}));
+    auto run = [&](uint64_t elements, uint64_t left) { return std::min(elements / bound, n_tiles / left); };
+    const uint64_t eight_waves = run(bound < 2048 || bound >= 3500 ? 16384 : 32768, 8 * 608);
+    const uint64_t r = bound < 3500 ? std::max(run(16384, 500), eight_waves) : eight_waves;
+    u.run = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(r, 1), 32);
   }
   u.n_units = (uint32_t)(u.run > 1 ? (n_tiles + u.run - 1) / u.run : n_tiles << u.log_parts);
   return u;

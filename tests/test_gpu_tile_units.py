@@ -69,6 +69,8 @@ CASES = [
     # short tiles in runs: joined, with gaps between ranges, single elements
     (120_000, [(0, 120_000)], 100), (130_000, [(k * 130 + k % 3, k * 130 + 97) for k in range(1000)], 32),
     (70_000, [(1, 69_999)], 16), (6_000, [(2 * k, 2 * k + 1) for k in range(3000)], 4),
+    # a third of the arena: shorter tiles than the bound says
+    (5_000_000, [(3_300_001, 4_966_668)], 1000),
     # more units than three waves: taken over early and late
     (2048 * 8000, [(2, 2048 * 8000)], 2_048),
 ]
