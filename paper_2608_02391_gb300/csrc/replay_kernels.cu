@@ -169,8 +169,25 @@ __device__ __forceinline__ void replay_stream(const ReplayArgs &r, uint64_t n_al
 template <int OP>
 constexpr uint32_t replay_tag() { return OP == kOpInit ? COPES_TAG_INIT : COPES_TAG_NOISE; }
 
+// A member's noise word, for any counter.
+template <int OP>
+__device__ __forceinline__ uint32_t replay_word(const ElemArgs &a, uint64_t g) {
+  uint32_t x[4];
+  philox4x32_10_rk((uint32_t)(g >> 2), (uint32_t)(g >> 34), 0u, replay_tag<OP>(), a.rk, x);
+  const uint32_t sel = (uint32_t)g & 3u;
+  return sel == 0 ? x[0] : (sel == 1 ? x[1] : (sel == 2 ? x[2] : x[3]));
+}
+template <int OP>
+static __device__ __noinline__ uint32_t replay_word_high(const ElemArgs &a, uint64_t g) {
+  return replay_word<OP>(a, g);
+}
+
 // Perturb / restore / commit / init over the members of the block's hash tiles: four
-// members per lane per batch, their master loads issued together.
+// members per lane per batch, their master loads issued together.  The hashing variant is
+// bound by its instructions: a batch's noise is formed together, from one word of a Philox
+// block each, whether or not a member is to be stored (perturb of 16.8M members of 2^28
+// elements 370 -> 336 us).  The mask variant is bound by scattered sectors and keeps fewer
+// registers instead (pair 373 us, 378 with single words).
 template <int OP, typename WT, bool MASK>
 __global__ void __launch_bounds__(kThreads) replay_elem_kernel(const __grid_constant__ ElemArgs a,
                                                                const __grid_constant__ ReplayArgs r) {
@@ -201,6 +218,21 @@ __global__ void __launch_bounds__(kThreads) replay_elem_kernel(const __grid_cons
       }
       th[u] = (OP != kOpInit && OP != kOpPartner && ok[u]) ? master[g[u]] : 0.0f;
     }
+    float eps[U];
+    if constexpr (kNoise && !MASK) {
+      uint32_t wd[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint64_t m = (uint64_t)kPhiloxM0 * (uint32_t)(g[u] >> 2);
+        const bool h = (uint32_t)g[u] & 2u, odd = (uint32_t)g[u] & 1u;
+        wd[u] = a.n_alloc > 1ull << 34
+                    ? replay_word_high<OP>(a, g[u])
+                    : philox4x32_10_word((uint32_t)m, (uint32_t)(m >> 32), a.fk, h, odd, h ? a.rk[16] : a.rk[17],
+                                         h ? a.rk[19] : a.rk[18]);
+      }
+#pragma unroll
+      for (int u = 0; u < U; u += 2) unpack_f32x2(normal_pair(wd[u], wd[u + 1], tab), eps[u], eps[u + 1]);
+    }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (!ok[u]) continue;
@@ -209,17 +241,12 @@ __global__ void __launch_bounds__(kThreads) replay_elem_kernel(const __grid_cons
         continue;
       }
       float v, vp = 0.0f;
-      if (OP == kOpRestore) {
+      if constexpr (OP == kOpRestore) {
         v = th[u];
       } else {
-        uint32_t x[4];
-        const uint64_t q = g[u] >> 2;
-        philox4x32_10_rk((uint32_t)q, (uint32_t)(q >> 32), 0u, replay_tag<OP>(), a.rk, x);
-        const uint32_t sel = (uint32_t)g[u] & 3u;
-        const uint32_t wd = sel == 0 ? x[0] : (sel == 1 ? x[1] : (sel == 2 ? x[2] : x[3]));
-        const float eps = normal_from_word(wd, tab);
-        v = __fmaf_rn(a.a, eps, OP == kOpInit ? a.b : th[u]);
-        if (OP == kOpPerturbPair) vp = __fmaf_rn(-a.a, eps, th[u]);
+        if (MASK) eps[u] = normal_from_word(replay_word<OP>(a, g[u]), tab);
+        v = __fmaf_rn(a.a, eps[u], OP == kOpInit ? a.b : th[u]);
+        if (OP == kOpPerturbPair) vp = __fmaf_rn(-a.a, eps[u], th[u]);
         if (OP == kOpInit) master[g[u]] = v;
       }
       WStore<WT>::one(a.w, g[u], v);

@@ -210,3 +210,28 @@ def test_membership_mask_equals_hashing(copes, layout, K, k):
     copes.perturb(a1, s1, 5, 1e-3)
     assert np.array_equal(w_bits(a1), w_bits(a2))
     copes.check()
+
+
+def test_hashing_past_counter_2_32_equals_the_mask(copes):
+    """An arena with indices from 2^34 on: the hashing kernels' noise comes from whole
+    Philox calls there instead of single words, as the mask's always does."""
+    lo, n = 1 << 34, (1 << 34) + 70_001
+    lay = copes.Layout([1 << 34, n - lo])
+    a = copes.Arena(torch.zeros(n, dtype=torch.bfloat16, device="cuda"), torch.zeros(n, device="cuda"))
+    a.master[lo - 70_000:] = torch.randn(n - lo + 70_000, device="cuda")
+    sub = copes.hash_replay_partition(lay, 16, 77)[3]
+    part = slice(lo - 70_000, n)
+    buf = torch.zeros(n, dtype=torch.bfloat16, device="cuda")
+
+    def step():
+        a.w.zero_(), buf.zero_()
+        copes.perturb(a, sub, 5, 1e-1)
+        out = [a.w[part].clone()]
+        copes.perturb_pair(a, sub, 6, 1e-1, buf)
+        return out + [a.w[part].clone(), buf[part].clone()]
+
+    got = step()
+    copes.hash_replay_mask(a, sub)
+    for x, y in zip(got, step()):
+        assert x.count_nonzero() > 70_000 // 16 and torch.equal(x, y)
+    copes.check()
