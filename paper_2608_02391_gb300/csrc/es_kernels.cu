@@ -348,8 +348,8 @@ __global__ void __launch_bounds__(kThreads, 3) restore_tiles_kernel(const __grid
 }
 
 // The partner member's perturb over TILES: w[g] = partner[g - partner_base], a copy of
-// the working dtype's bits (the values kOpPerturbPair wrote).  Aligned stretches move one
-// 4-element group (8 B bf16, 16 B fp32) per load; others go element by element.
+// the working dtype's bits (the values kOpPerturbPair wrote), by whole 4-element groups (8 B
+// bf16, 16 B fp32); partner_base is a multiple of 4, so both sides' groups are aligned.
 template <typename WT>
 struct Group4;
 template <>
@@ -365,25 +365,24 @@ template <typename WT, int G>
 __global__ void __launch_bounds__(kThreads) partner_tiles_kernel(const __grid_constant__ ElemArgs a) {
   for_unit(blockIdx.x, a.units, a.tiles, a.n_tiles, a.n_alloc, flag_error,
            [&](uint64_t b, uint64_t e) { return partner_covers(a, b, e); }, [&](uint64_t b, uint64_t e) {
-    const WT *__restrict__ src = reinterpret_cast<const WT *>(a.partner) + (b - a.partner_base);
-    WT *__restrict__ dst = reinterpret_cast<WT *>(a.w) + b;
-    const uint32_t len = (uint32_t)(e - b);
-    if (((b | e) & 3ull) == 0) {  // partner_base is a multiple of 4, so src is aligned too
-      using V = typename Group4<WT>::T;
-      const V *__restrict__ vs = reinterpret_cast<const V *>(src);
-      V *__restrict__ vd = reinterpret_cast<V *>(dst);
-      const uint32_t n = len / 4;
-      for (uint32_t i0 = threadIdx.x; i0 < n; i0 += kThreads * G) {
-        V v[G];
+    const uint64_t lo = (b + 3) & ~3ull, hi = e & ~3ull;  // the whole groups, if lo < hi
+    const WT *__restrict__ src = reinterpret_cast<const WT *>(a.partner);
+    WT *__restrict__ dst = reinterpret_cast<WT *>(a.w);
+    const uint64_t edge = threadIdx.x < 4 ? b + threadIdx.x : hi + threadIdx.x - 4;
+    if (threadIdx.x < 8 && edge < e && (threadIdx.x < 4 ? edge < lo : hi >= lo)) dst[edge] = src[edge - a.partner_base];
+    if (lo >= hi) return;
+    using V = typename Group4<WT>::T;
+    const V *__restrict__ vs = reinterpret_cast<const V *>(src + (lo - a.partner_base));
+    V *__restrict__ vd = reinterpret_cast<V *>(dst + lo);
+    const uint32_t n = (uint32_t)(hi - lo) / 4;
+    for (uint32_t i0 = threadIdx.x; i0 < n; i0 += kThreads * G) {
+      V v[G];
 #pragma unroll
-        for (int k = 0; k < G; ++k)
-          if (i0 + kThreads * k < n) v[k] = __ldcs(vs + i0 + kThreads * k);
+      for (int k = 0; k < G; ++k)
+        if (i0 + kThreads * k < n) v[k] = __ldcs(vs + i0 + kThreads * k);
 #pragma unroll
-        for (int k = 0; k < G; ++k)
-          if (i0 + kThreads * k < n) __stcs(vd + i0 + kThreads * k, v[k]);
-      }
-    } else {
-      for (uint32_t i = threadIdx.x; i < len; i += kThreads) dst[i] = src[i];
+      for (int k = 0; k < G; ++k)
+        if (i0 + kThreads * k < n) __stcs(vd + i0 + kThreads * k, v[k]);
     }
   });
 }
@@ -484,7 +483,10 @@ static cudaError_t launch_elem_typed(int kind, ElemArgs &a, cudaStream_t s) {
     if (kind == COPES_SUBSPACE_TILES) {
       if (OP == kOpPerturbTwoPairs && a.copies.n != 3) return cudaErrorInvalidValue;
       if (a.n_tiles == 0) return cudaSuccess;
-      a.units = plan_tile_units(a.n_tiles, a.n_alloc, 2, 1216);
+      // a copy, or a restore of one or two, has too little to do for parts beyond one tile an SM:
+      // 4M elements 5.4 us whole, 6.8 in quarters (restore of one), 11.1M 12.5 and 14.8
+      const bool light = OP == kOpPartner || (OP == kOpRestore && a.copies.n <= 1);
+      a.units = plan_tile_units(a.n_tiles, a.n_alloc, 2, light ? 152 : 1216);
       const unsigned grid = a.units.n_units;
       if constexpr (OP == kOpPartner) partner_tiles_kernel<WT, 8><<<grid, kThreads, 0, s>>>(a);
       else if constexpr (OP == kOpRestore) restore_tiles_kernel<WT, 8><<<grid, kThreads, 0, s>>>(a);
@@ -683,13 +685,32 @@ __global__ void __launch_bounds__(kThreads) update_index_kernel(const __grid_con
   });
 }
 
+// log2 of the parts an update cuts its tiles into.  Up to 128 tiles, sixteenths (one group a
+// thread).  Up to eight waves the SM with the most parts sets the time: of the cuts that give
+// each SM its four blocks, the one with the least ceil(parts / 152) (1 / 2^log + overhead / P),
+// the overhead of a part being a fifth of a tile's time for one noise vector.  With up to three
+// noise vectors the update is bound by memory and whole tiles are best.  Start / eighths up to
+// 608 tiles and whole ones above / this, us: P = 16, 3M, 6M, 11.1M and 18M elements 84.6 /
+// 51.2 / 49.2, 122.6 / 93.8 / 91.5, 196 / 176 / 155 and 306 / 272 / 266; P = 4, 8M 48.0 / 47.8 /
+// 44.0; P = 1, 8M 26.1 / 40.6 / 27.5.
+static uint32_t update_log_parts(uint64_t n_tiles, int n_noise) {
+  if (n_tiles <= (n_noise <= 3 ? 192u : 128u)) return 4;
+  if (n_noise <= 3 || n_tiles > 8 * 152) return 0;
+  uint32_t best = 0;
+  double best_cost = 1e30;
+  for (uint32_t log = 0; log <= 3; ++log) {
+    if ((n_tiles << log) < 4 * 152) continue;
+    const double cost = (double)(((n_tiles << log) + 151) / 152) * (1.0 / (1 << log) + 0.2 / n_noise);
+    if (cost < best_cost) best = log, best_cost = cost;
+  }
+  return best;
+}
+
 template <typename WT, bool COMMIT>
 static cudaError_t launch_update_typed(int kind, UpdateArgs &a, cudaStream_t s) {
   if (kind == COPES_SUBSPACE_TILES) {
     if (a.n_tiles == 0) return cudaSuccess;
-    // sixteenths (one group a thread) while they are at most 3.4 waves, else eighths: P = 32, 2^18,
-    // 2^20 and 4M elements 14.3 / 13.7, 38.8 / 36.6 and 121.8 / 125.1 us (eighths / sixteenths)
-    a.units = plan_tile_units(a.n_tiles, a.n_alloc, a.n_tiles <= 128 ? 4 : 3, 608);
+    a.units = plan_tile_units(a.n_tiles, a.n_alloc, update_log_parts(a.n_tiles, a.n_noise), 8 * 152 + 1);
     update_tiles_kernel<WT, kUpdateGroups, COMMIT, kUpdateBlocksPerSM>
         <<<a.units.n_units, kThreads, update_smem_bytes(a.n_noise), s>>>(a);
   } else {
