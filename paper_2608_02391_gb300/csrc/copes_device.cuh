@@ -181,6 +181,7 @@ __device__ __forceinline__ void ld_stream_f8(const float *p, float (&x)[4], floa
                : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(y[0]), "=f"(y[1]), "=f"(y[2]), "=f"(y[3])
                : "l"(p));
 }
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void st_stream_f4(float *p, float4 v) {
   __stcs(reinterpret_cast<float4 *>(p), v);
 }

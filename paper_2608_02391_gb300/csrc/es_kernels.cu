@@ -532,10 +532,14 @@ cudaError_t launch_elementwise(int op, int kind, int dtype, ElemArgs &a, cudaStr
 // (noise_sum_groups), acc = sum_j w_j eps_j (j ascending), and writes theta = fma(coef, acc,
 // theta) and, with COMMIT, its rounding to the working copies.  All counters of [b, e) have
 // the high word s.q_hi.
-template <typename WT, int G, bool COMMIT>
+template <typename WT, int G, bool COMMIT, bool AHEAD>
 __device__ __forceinline__ void update_step(const UpdateArgs &a, const UpdateSmem &s, uint64_t base, uint64_t b,
                                             uint64_t e) {
   float *__restrict__ master = a.master;
+  if (AHEAD)
+#pragma unroll
+    for (int i = 0; i < G; ++i)
+      if (base + 4ull * kThreads * i < e) prefetch_l2(master + base + 4ull * kThreads * i);
   float acc[G][4];
   noise_sum_groups<G>(base, a.n_noise, s, acc);
   // theta is read only now, after the noise loop, so it occupies no registers there
@@ -570,24 +574,24 @@ __device__ __forceinline__ void update_step(const UpdateArgs &a, const UpdateSme
 }
 
 // Steps of G groups while they are whole for the block, then of single groups.
-template <typename WT, int G, bool COMMIT>
+template <typename WT, int G, bool COMMIT, bool AHEAD>
 __device__ __forceinline__ void update_range(const UpdateArgs &a, const UpdateSmem &s, uint64_t b, uint64_t e,
                                              NextUnit &next) {
   constexpr uint64_t kStep = 4ull * kThreads * G;
   uint64_t at = b & ~3ull;
   for (; at + kStep <= e; at += kStep) {
     if (at + 2 * kStep > e) next.ask();
-    update_step<WT, G, COMMIT>(a, s, at + 4ull * threadIdx.x, b, e);
+    update_step<WT, G, COMMIT, AHEAD>(a, s, at + 4ull * threadIdx.x, b, e);
   }
   for (uint64_t base = at + 4ull * threadIdx.x; base < e; base += 4ull * kThreads)
-    update_step<WT, 1, COMMIT>(a, s, base, b, e);
+    update_step<WT, 1, COMMIT, AHEAD>(a, s, base, b, e);
 }
 
 // update_range for exactly kUpdateSpan elements from an aligned b (the default tile size),
 // with compile-time bounds and no edge tests: the same values bit for bit.
 constexpr uint32_t kUpdateSpan = 16384;
 
-template <typename WT, int G, bool COMMIT>
+template <typename WT, int G, bool COMMIT, bool AHEAD>
 __device__ __forceinline__ void update_span(const UpdateArgs &a, const UpdateSmem &s, uint64_t b, NextUnit &next) {
   constexpr uint32_t kStep = 4u * kThreads * G;
   static_assert(kUpdateSpan % kStep == 0, "a full span is whole steps");
@@ -595,6 +599,13 @@ __device__ __forceinline__ void update_span(const UpdateArgs &a, const UpdateSme
   for (uint32_t at = 0; at < kUpdateSpan; at += kStep) {
     if (at == kUpdateSpan - kStep) next.ask();
     const uint32_t off = at + 4u * threadIdx.x;
+    if (AHEAD)
+#pragma unroll
+      for (int i = 0; i < G; ++i) {
+        const float *t = mt + off + 4u * kThreads * i;
+        if (at == 0) prefetch_l2(t);
+        if (at + kStep < kUpdateSpan) prefetch_l2(t + kStep);
+      }
     float acc[G][4];
     noise_sum_groups<G>(b + off, a.n_noise, s, acc);
 #pragma unroll
@@ -619,7 +630,13 @@ __device__ __forceinline__ void update_span(const UpdateArgs &a, const UpdateSme
 constexpr int kUpdateGroups = 2;
 constexpr int kUpdateBlocksPerSM = 4;
 
-template <typename WT, int G, bool COMMIT, int BLOCKS>
+// AHEAD: theta is asked into L2 a step ahead of its noise, which costs no registers.  Few noise
+// vectors do not hide its latency: 134M elements, P = 1, 2, 4 and 8 355 -> 327, 385 -> 329,
+// 522 -> 498 and 946 -> 922 us.  With more it gains nothing (P = 16 1,776 / 1,782), and the form
+// without it is the faster code.
+constexpr int kAheadNoise = 8;
+
+template <typename WT, int G, bool COMMIT, int BLOCKS, bool AHEAD>
 __global__ void __launch_bounds__(kThreads, BLOCKS) update_tiles_kernel(const __grid_constant__ UpdateArgs a) {
   extern __shared__ __align__(128) char s_update[];
   __shared__ UnitSmem s_unit;
@@ -631,8 +648,8 @@ __global__ void __launch_bounds__(kThreads, BLOCKS) update_tiles_kernel(const __
       while (b < e) {  // one pass, two where the counters' high word changes
         const uint64_t end = min(e, ((b >> 34) + 1) << 34);
         update_keys_for(a, s, b);
-        if (end - b == kUpdateSpan && (b & 3ull) == 0) update_span<WT, G, COMMIT>(a, s, b, next);
-        else update_range<WT, G, COMMIT>(a, s, b, end, next);
+        if (end - b == kUpdateSpan && (b & 3ull) == 0) update_span<WT, G, COMMIT, AHEAD>(a, s, b, next);
+        else update_range<WT, G, COMMIT, AHEAD>(a, s, b, end, next);
         b = end;
       }
     });
@@ -686,22 +703,27 @@ __global__ void __launch_bounds__(kThreads) update_index_kernel(const __grid_con
 }
 
 // log2 of the parts an update cuts its tiles into.  Up to 128 tiles, sixteenths (one group a
-// thread).  Up to eight waves the SM with the most parts sets the time: of the cuts that give
-// each SM its four blocks, the one with the least ceil(parts / 152) (1 / 2^log + overhead / P),
-// the overhead of a part being a fifth of a tile's time for one noise vector.  With up to three
-// noise vectors the update is bound by memory and whole tiles are best.  Start / eighths up to
-// 608 tiles and whole ones above / this, us: P = 16, 3M, 6M, 11.1M and 18M elements 84.6 /
-// 51.2 / 49.2, 122.6 / 93.8 / 91.5, 196 / 176 / 155 and 306 / 272 / 266; P = 4, 8M 48.0 / 47.8 /
-// 44.0; P = 1, 8M 26.1 / 40.6 / 27.5.
+// thread).  Beyond, of the cuts that give each SM its four blocks, the one with the least
+// ceil(parts / slots) (1 / 2^log + overhead / P), the overhead of a part being a fifth to a third of
+// a tile's time for one noise vector: up to two waves of tiles the SM with the most parts sets
+// the time (152 slots), beyond the last wave does (608), where parts have to gain 3%.  With up
+// to three noise vectors the update is bound by memory and whole tiles are best, as they are
+// with four beyond two waves.  Start / eighths up to 608 tiles and whole ones above / this, us:
+// P = 16, 3M, 6M, 11.1M and 18M elements 84.6 / 51.2 / 49.2, 122.6 / 93.8 / 91.5, 196 / 176 /
+// 155 and 306 / 272 / 266; P = 4, 8M 48.0 / 47.8 / 39.3; P = 1, 8M 26.1 / 40.6 / 26.5; P = 64,
+// 30M and 134M 1,900 / 1,670 / 1,574 and 7,820 / 7,066 / 6,867.
 static uint32_t update_log_parts(uint64_t n_tiles, int n_noise) {
   if (n_tiles <= (n_noise <= 3 ? 192u : 128u)) return 4;
-  if (n_noise <= 3 || n_tiles > 8 * 152) return 0;
+  const bool waves = n_tiles > 8 * 152;
+  if (n_noise <= (waves ? 4 : 3)) return 0;
+  const uint64_t slots = waves ? 4 * 152 : 152;
+  const double overhead = (waves ? 0.3 : 0.2) / n_noise;
   uint32_t best = 0;
   double best_cost = 1e30;
-  for (uint32_t log = 0; log <= 3; ++log) {
+  for (uint32_t log = 0; log <= (waves ? 2u : 3u); ++log) {
     if ((n_tiles << log) < 4 * 152) continue;
-    const double cost = (double)(((n_tiles << log) + 151) / 152) * (1.0 / (1 << log) + 0.2 / n_noise);
-    if (cost < best_cost) best = log, best_cost = cost;
+    const double cost = (double)(((n_tiles << log) + slots - 1) / slots) * (1.0 / (1 << log) + overhead);
+    if (cost < best_cost * (waves && best == 0 ? 0.97 : 1.0)) best = log, best_cost = cost;
   }
   return best;
 }
@@ -710,9 +732,11 @@ template <typename WT, bool COMMIT>
 static cudaError_t launch_update_typed(int kind, UpdateArgs &a, cudaStream_t s) {
   if (kind == COPES_SUBSPACE_TILES) {
     if (a.n_tiles == 0) return cudaSuccess;
-    a.units = plan_tile_units(a.n_tiles, a.n_alloc, update_log_parts(a.n_tiles, a.n_noise), 8 * 152 + 1);
-    update_tiles_kernel<WT, kUpdateGroups, COMMIT, kUpdateBlocksPerSM>
-        <<<a.units.n_units, kThreads, update_smem_bytes(a.n_noise), s>>>(a);
+    a.units = plan_tile_units(a.n_tiles, a.n_alloc, update_log_parts(a.n_tiles, a.n_noise), ~0u);
+    auto kernel = a.n_noise <= kAheadNoise
+                      ? update_tiles_kernel<WT, kUpdateGroups, COMMIT, kUpdateBlocksPerSM, true>
+                      : update_tiles_kernel<WT, kUpdateGroups, COMMIT, kUpdateBlocksPerSM, false>;
+    kernel<<<a.units.n_units, kThreads, update_smem_bytes(a.n_noise), s>>>(a);
   } else {
     if (a.n_index == 0) return cudaSuccess;
     a.segment = index_segment(a.n_index);

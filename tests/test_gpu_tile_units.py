@@ -121,3 +121,22 @@ def test_two_pairs_over_whole_tiles_equal_pairs(copes, begin, offset):
         copes.perturb_pair(a, sub, seed, 1e-3, a.w2)
         assert torch.equal(a.w, got[2 * k]) and torch.equal(a.w2, got[2 * k + 1])
     copes.check()
+
+
+@pytest.mark.parametrize("tiles", [130, 187, 679, 1217, 1860])
+@pytest.mark.parametrize("P", [4, 8, 9, 40])
+def test_update_cuts_equal_the_index_list(copes, P, tiles):
+    """Tile counts and noise vectors at which the update's tiles are cut differently, and on both
+    sides of the count up to which theta is asked for ahead."""
+    begin, size = 6, 9_000  # longer than half the default tile, so that tiles are not joined
+    n = begin + tiles * size - 777
+    nid, sign, _ = copes.member_table(2 * P, copes.ANTITHETIC)
+    f = torch.linspace(-1, 1, 2 * P, device="cuda")
+    got = []
+    for sub in (copes.tiles_from_ranges([(begin, n)], tile_size=size), index_list(copes, [(begin, n)])):
+        a = arena(copes, n, torch.bfloat16)
+        copes.update(a, sub, nid, sign, f, copes.member_seeds(33, 1, 2, P), 1e-2)
+        got.append([a.master] + a.copies)
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
+    copes.check()
