@@ -65,14 +65,14 @@ FALLBACK_HBM_GBS = 6800.0
 # subspaces of 2^28 parameters, where the writes still in L2 when the kernel ends are at most
 # 2% of its traffic.
 NCU_TRAFFIC = {
-    "perturb_two_pairs": {"kernel": "elem_tiles_kernel<perturb_two_pairs,bf16>", "source_sha": "9924be7439c3aa0f",
-                          "bytes_per_elem": 11.943, "capture": "profiles/perturb_two_pairs_4b_slice.md",
+    "perturb_two_pairs": {"kernel": "elem_tiles_kernel<perturb_two_pairs,bf16>", "source_sha": "0dc5faba317930d4",
+                          "bytes_per_elem": 11.945, "capture": "profiles/perturb_two_pairs_4b_slice.md",
                           "case": "two 2^28-parameter subspaces (--case 4b-slice-big)"},
-    "perturb_pair": {"kernel": "elem_tiles_kernel<perturb_pair,bf16>", "source_sha": "9924be7439c3aa0f",
+    "perturb_pair": {"kernel": "elem_tiles_kernel<perturb_pair,bf16>", "source_sha": "0dc5faba317930d4",
                      "bytes_per_elem": 7.846, "capture": "profiles/perturb_pair_4b_slice.md",
                      "case": "two 2^28-parameter subspaces (--case 4b-slice-big --weights dual)"},
-    "perturb": {"kernel": "elem_tiles_kernel<perturb,bf16>", "source_sha": "9924be7439c3aa0f",
-                "bytes_per_elem": 5.877, "capture": "profiles/perturb_4b_slice.md",
+    "perturb": {"kernel": "elem_tiles_kernel<perturb,bf16>", "source_sha": "0dc5faba317930d4",
+                "bytes_per_elem": 5.876, "capture": "profiles/perturb_4b_slice.md",
                 "case": "two 2^28-parameter subspaces (--case 4b-slice-big --weights single)"},
 }
 

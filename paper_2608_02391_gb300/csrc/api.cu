@@ -23,10 +23,9 @@ using copes::UpdateArgs;
 // here (disjoint tiles: n_alloc / n_tiles), so no part is made shorter than 1,024 elements
 // by that bound; a part of a tile that turns out shorter may come out empty.
 // Measured (bf16, 16,384-element tiles; start / one unit a tile / these parts): the
-// two-pairs perturb of 2^18, 2^20 and 14.9M elements 7.6 / 7.5 / 2.9, 8.0 / 7.8 / 4.5 and
-// 39.2 / 36.5 / 36.3 us; the update (P = 16) of 2^18, 2^20 and 4M elements 47.8 / 46.0 /
-// 9.3, 47.9 / 46.2 / 21.5 and 85.3 / 79.8 / 62.9 us, of 14.9M elements 234 / 215 / 221 us;
-// tiles of 1,000 elements joined, 11.1M elements: perturb 29.0 -> 18.8 us, update 351 -> 178.
+// two-pairs perturb of 2^18, 2^20 and 14.9M elements 7.6 / 7.5 / 3.3, 8.0 / 7.8 / 4.5 and
+// 39.2 / 36.5 / 34.1 us; tiles of 1,000 elements joined, 11.1M elements: perturb 29.0 -> 18.8
+// us, update (P = 16) 351 -> 176.  The update brings its own cut (log_parts).
 // The bound is loose by as much as the subspace is a part of the arena, and a run then holds
 // less than it says: short tiles are joined while 500 units are left, and those of a middling
 // bound up to 32,768 elements by it while there are eight waves of units.  Tiles of 1,000 in a
@@ -38,7 +37,7 @@ copes::TileUnits copes::plan_tile_units(uint64_t n_tiles, uint64_t n_alloc, uint
   TileUnits u{(uint32_t)n_tiles, 0, 1};
   const uint64_t bound = std::max<uint64_t>(1, n_alloc / n_tiles);  // >= the mean tile length
   if (bound > 8192) {
-    if (n_tiles < few) u.log_parts = log_parts;
+    if (n_tiles < few && n_tiles < 1u << 24) u.log_parts = log_parts;  // the grid stays in 32 bits
   } else if (n_tiles < 500) {
     while ((n_tiles << (u.log_parts + 1)) <= 500 && (bound >> (u.log_parts + 1)) >= 1024) ++u.log_parts;
   } else {
