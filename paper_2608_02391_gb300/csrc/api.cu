@@ -22,7 +22,7 @@ using copes::UpdateArgs;
 // instead, while enough units are left.  Only a bound of the mean tile length is known
 // here (disjoint tiles: n_alloc / n_tiles), so no part is made shorter than 1,024 elements
 // by that bound; a part of a tile that turns out shorter may come out empty.
-// Measured (bf16, 16,384-element tiles; start / one unit a tile / these parts): the
+// Measured (bf16, 16,384-element tiles; one block a tile / one unit a tile / these parts): the
 // two-pairs perturb of 2^18, 2^20 and 14.9M elements 7.6 / 7.5 / 3.3, 8.0 / 7.8 / 4.5 and
 // 39.2 / 36.5 / 34.1 us; tiles of 1,000 elements joined, 11.1M elements: perturb 29.0 -> 18.8
 // us, update (P = 16) 351 -> 176.  The update brings its own cut (log_parts).

@@ -708,7 +708,7 @@ __global__ void __launch_bounds__(kThreads) update_index_kernel(const __grid_con
 // a tile's time for one noise vector: up to two waves of tiles the SM with the most parts sets
 // the time (152 slots), beyond the last wave does (608), where parts have to gain 3%.  With up
 // to three noise vectors the update is bound by memory and whole tiles are best, as they are
-// with four beyond two waves.  Start / eighths up to 608 tiles and whole ones above / this, us:
+// with four beyond two waves.  A block a tile / eighths to 608 tiles, whole ones above / this, us:
 // P = 16, 3M, 6M, 11.1M and 18M elements 84.6 / 51.2 / 49.2, 122.6 / 93.8 / 91.5, 196 / 176 /
 // 155 and 306 / 272 / 266; P = 4, 8M 48.0 / 47.8 / 39.3; P = 1, 8M 26.1 / 40.6 / 26.5; P = 64,
 // 30M and 134M 1,900 / 1,670 / 1,574 and 7,820 / 7,066 / 6,867.

@@ -235,3 +235,23 @@ def test_hashing_past_counter_2_32_equals_the_mask(copes):
     for x, y in zip(got, step()):
         assert x.count_nonzero() > 70_000 // 16 and torch.equal(x, y)
     copes.check()
+
+
+@pytest.mark.parametrize("tiles", [1, 5, 607, 1216, 1300, 1830, 2433])
+def test_any_number_of_hash_tiles_equals_the_lists(copes, tiles):
+    """The kernels' blocks take 1 to 4 consecutive hash tiles, by the number of tiles."""
+    n, K, k = tiles * 16_384 - 1_000, 16, 7
+    lay = copes.Layout([n])
+    theta = torch.randn(n, device="cuda")
+    out = []
+    for sub in (copes.hash_replay_partition(lay, K, 77)[k], copes.hash_partition(lay, K, 77)[k]):
+        a = copes.Arena(torch.zeros(n, dtype=torch.bfloat16, device="cuda"), theta.clone())
+        copes.perturb(a, sub, 5, 1e-1)
+        got = [a.w.clone()]
+        nid, sign, P = copes.member_table(6, copes.ANTITHETIC)
+        f = torch.linspace(-1, 1, 6, device="cuda")
+        copes.update(a, sub, nid, sign, f, copes.member_seeds(33, 1, 2, P), 1e-2)
+        out.append(got + [a.w, a.master])
+    for x, y in zip(*out):
+        assert torch.equal(x, y)
+    copes.check()
