@@ -271,11 +271,14 @@ struct UpdateArgs {
 };
 
 // ------------------------------------------------------------------------ launchers
-// Lets `kernel` take `dynamic` bytes of dynamic shared memory when that and its static share
-// pass the default limit of 48 KB a block (host).
-inline cudaError_t allow_smem(const void *kernel, uint32_t total, uint32_t dynamic) {
+// Lets `kernel` be launched with `total` bytes of shared memory, its static share among them,
+// when that is past the default limit of 48 KB a block (host).  The limit belongs to the kernel
+// on this device, for every thread of the process: it is set to `most`, the most dynamic
+// shared memory that any call takes, so that no call lowers it between another thread's
+// setting and its launch.
+inline cudaError_t allow_smem(const void *kernel, uint32_t total, uint32_t most) {
   if (total <= 48u * 1024u) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic);
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
 // The units of a launch over n_tiles disjoint tiles of an n_alloc-element arena (n_tiles in

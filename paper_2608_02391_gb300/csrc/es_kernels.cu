@@ -743,7 +743,7 @@ static cudaError_t launch_update_typed(int kind, UpdateArgs &a, cudaStream_t s) 
     const unsigned blocks = (unsigned)((a.n_index + a.segment - 1) / a.segment);
     const uint32_t smem = gather_smem_bytes(a.n_noise);
     auto kernel = a.gathered ? update_index_kernel<WT, COMMIT, true> : update_index_kernel<WT, COMMIT, false>;
-    const cudaError_t e = allow_smem((const void *)kernel, smem + 2 * kStageChunk * 8 + 64, smem);
+    const cudaError_t e = allow_smem((const void *)kernel, smem + 2 * kStageChunk * 8 + 64, gather_smem_bytes(COPES_MAX_NOISE));
     if (e != cudaSuccess) return e;
     kernel<<<blocks, kThreads, smem, s>>>(a);
   }

@@ -343,7 +343,7 @@ cudaError_t launch_hash_scatter(const HashTensor *tensors, int n_tensors, uint64
   ListTable t;
   for (int k = 0; k < COPES_MAX_K; ++k) t.list[k] = k < K ? lists[k] : nullptr;
   const uint32_t smem = kScatterSmem(K);
-  const cudaError_t e = allow_smem((const void *)hash_scatter_kernel, smem + 1024, smem);
+  const cudaError_t e = allow_smem((const void *)hash_scatter_kernel, smem + 1024, kScatterSmem(COPES_MAX_K));
   if (e != cudaSuccess) return e;
   hash_scatter_kernel<<<(unsigned)n_htiles, kPartThreads, smem, s>>>(tensors, n_tensors, K, seed, offsets, t);
   return cudaGetLastError();

@@ -365,7 +365,8 @@ static cudaError_t launch_replay_update_typed(const UpdateArgs &a, const ReplayA
   if (r.n_tiles == 0) return cudaSuccess;
   const uint32_t smem = gather_smem_bytes(a.n_noise);
   auto kernel = r.mask ? replay_update_kernel<WT, COMMIT, true> : replay_update_kernel<WT, COMMIT, false>;
-  const cudaError_t e = allow_smem((const void *)kernel, smem + 16 * 1024, smem);  // 8.5 KB static
+  // 8.5 KB static
+  const cudaError_t e = allow_smem((const void *)kernel, smem + 16 * 1024, gather_smem_bytes(COPES_MAX_NOISE));
   if (e != cudaSuccess) return e;
   kernel<<<replay_blocks(r.n_tiles), kThreads, smem, s>>>(a, r);
   return cudaGetLastError();
