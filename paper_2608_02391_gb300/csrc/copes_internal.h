@@ -198,6 +198,20 @@ struct TileUnits {
   uint32_t n_units, log_parts, run;
 };
 
+// Whether [b, e), as read from a device tile table, is a tile of the arena.  The kernels touch
+// nothing of a tile before this has held: e - b alone says nothing of a tile with b > e,
+// where it wraps.
+__host__ __device__ __forceinline__ bool tile_in_arena(uint64_t b, uint64_t e, uint64_t n_alloc) {
+  return b <= e && e <= n_alloc && e - b <= (uint64_t)COPES_TILE_MAX;
+}
+
+// Whether the tile [b, e) is in the arena and its 2^log_parts parts are `part` whole groups'
+// elements each, all with counters below 2^32.
+__host__ __device__ __forceinline__ bool tile_in_whole_parts(uint64_t b, uint64_t e, uint64_t n_alloc, uint32_t part,
+                                                             uint32_t log_parts) {
+  return tile_in_arena(b, e, n_alloc) && e - b == (uint64_t)part << log_parts && (b & 3) == 0 && (e >> 34) == 0;
+}
+
 // The working copies beyond w (copes_params.w2, w3, w4): n = 0, 1 (w2) or 3 (w2, w3, w4).
 struct WorkingCopies {
   void *p[3];

@@ -96,7 +96,7 @@ __device__ __forceinline__ void for_unit(uint32_t unit, const TileUnits &u, cons
   const uint64_t first = (uint64_t)(unit >> u.log_parts) * u.run;
   const ulonglong2 *tab = reinterpret_cast<const ulonglong2 *>(tiles) + first;
   auto valid = [&](ulonglong2 v, bool reports) {
-    if (v.x > v.y || v.y > n_alloc || v.y - v.x > (uint64_t)COPES_TILE_MAX) {
+    if (!tile_in_arena(v.x, v.y, n_alloc)) {
       if (reports) flag(kErrTileRange);
       return false;
     }
@@ -142,7 +142,7 @@ __device__ __forceinline__ void prefetch_unit(const TileUnits &u, const uint64_t
   const ulonglong2 v =
       __ldg(reinterpret_cast<const ulonglong2 *>(tiles) + (uint64_t)(blockIdx.x >> u.log_parts) * u.run);
   uint64_t b = v.x, e = v.y;
-  if (b > e || e > n_alloc || e - b > (uint64_t)COPES_TILE_MAX) return;
+  if (!tile_in_arena(b, e, n_alloc)) return;
   if (u.log_parts) tile_part(u, blockIdx.x & ((1u << u.log_parts) - 1u), b, e);
   b &= ~3ull;  // 16-byte aligned; and whole 16 bytes
   const uint32_t bytes = (uint32_t)(e - b) * 4u & ~15u;

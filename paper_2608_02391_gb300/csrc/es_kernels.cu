@@ -284,7 +284,7 @@ __device__ __forceinline__ bool elem_part(const ElemArgs &a, const WideTable &ta
   const uint32_t lp = a.units.log_parts;
   if (a.units.run != 1) return false;
   const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(a.tiles) + (unit >> lp));
-  if (v.y - v.x != (uint64_t)(kElemPart << lp) || (v.x & 3) != 0 || v.y > a.n_alloc || (v.y >> 34) != 0) return false;
+  if (!tile_in_whole_parts(v.x, v.y, a.n_alloc, kElemPart, lp)) return false;
   if (OP == kOpPerturbPair && !(v.x >= a.partner_base && v.y - a.partner_base <= a.partner_len)) return false;
   next.ask();
   const uint64_t b = v.x + (unit - (unit >> lp << lp)) * kElemPart;

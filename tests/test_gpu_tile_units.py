@@ -105,6 +105,24 @@ def test_invalid_tile_in_a_run_is_left_out(copes):
     assert torch.equal(a.w, want)
 
 
+@pytest.mark.parametrize("size", [4096, 16_384])
+def test_reversed_tile_is_left_out(copes, size):
+    """A tile with b > e whose e - b wraps round to a whole part or tile."""
+    n = 4 * size
+    sub = copes.tiles_from_ranges([(0, n)], tile_size=size)
+    sub.tensor[1] = torch.tensor([-size, 0], device="cuda")  # [2^64 - size, 0)
+    a, b = arena(copes, n, torch.bfloat16), arena(copes, n, torch.bfloat16)
+    rest = index_list(copes, [(0, size), (2 * size, n)])
+    for x, s in ((a, sub), (b, rest)):
+        copes.perturb_pair(x, s, SEEDS[0], 1e-3, x.w2)
+    copes.restore(a, sub)
+    copes.restore(b, rest)
+    with pytest.raises(copes.CopesError) as e:
+        copes.check()
+    assert e.value.code == copes.ERR_DEVICE_CHECK and "0x1:" in str(e.value)
+    assert torch.equal(a.master, b.master) and all(torch.equal(x, y) for x, y in zip(a.copies, b.copies))
+
+
 @pytest.mark.parametrize("offset", [0, 4])  # floats before theta: 32-byte aligned or not
 @pytest.mark.parametrize("begin", [0, 4, 8, 3])
 def test_two_pairs_over_whole_tiles_equal_pairs(copes, begin, offset):
