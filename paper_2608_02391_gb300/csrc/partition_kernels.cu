@@ -108,33 +108,95 @@ __device__ __forceinline__ uint32_t warp_scan(uint32_t v) {
   return v;
 }
 
-// Block (k, c): exclusive prefix sum over tiles of hist[tile][k] -> offsets[tile][k] for the
-// tiles of chunk c, 4,096 of them, which it starts from the sum of all tiles before (its own
-// reads of them: no block waits for another).  One block per bucket for all tiles took
-// 39 us for 30,270 tiles and K = 16, bound by its SM's strided accesses.
+// The exclusive prefix sums of hist[tile][k] over the tiles, per bucket k, in chunks of 1,024
+// tiles.  Up to kScanReread chunks, a chunk's block sums the tiles before it itself; beyond,
+// two launches before it are linear in the tiles: the sums of the chunks, and their scan.
+// Until the last launch, the start of a chunk lies in offsets at the chunk's first tile,
+// which is where it belongs.  Re-read / with the launches before, us: 8,545 tiles, K = 16 and 64
+// 6.0 / 10.7 and 17 / 24; 12,208 tiles 10.2 / 12.3 and 28 / 26; 30,518 tiles 29 / 15 and 122 / 36;
+// 488,282 tiles 3,209 / 88 and 27,858 / 353.
 constexpr int kScanVec = 4;  // consecutive tiles a thread
-constexpr uint64_t kScanChunk = kScanVec * 1024;
+constexpr int kScanThreads = 256;
+constexpr uint64_t kScanChunk = kScanVec * kScanThreads;
+constexpr uint64_t kScanReread = 12;
+constexpr int kSumThreads = 1024;
+static_assert(kScanChunk * kHashTile < 1ull << 32, "a chunk's sum fits 32 bits");
+static_assert(COPES_MAX_K <= kSumThreads, "a thread per bucket");
 
-__global__ void __launch_bounds__(1024) hash_scan_kernel(const uint32_t *hist, uint64_t n_htiles,
-                                                         int K, uint64_t *offsets) {
-  __shared__ unsigned long long s_before[32];
-  __shared__ uint32_t s_warp[32];
+__global__ void __launch_bounds__(kSumThreads) hash_chunk_sums_kernel(const uint32_t *hist, uint64_t n_htiles, int K,
+                                                                       uint64_t *offsets) {
+  __shared__ uint32_t s_sum[COPES_MAX_K];
+  const uint64_t t0 = blockIdx.x * kScanChunk, rows = min(kScanChunk, n_htiles - t0);
+  if (threadIdx.x < K) s_sum[threadIdx.x] = 0;
+  __syncthreads();
+  const uint32_t at_once = kSumThreads / K, row = threadIdx.x / K, k = threadIdx.x % K;
+  uint32_t sum = 0;
+  if (row < at_once) {
+#pragma unroll 8
+    for (uint64_t r = row; r < rows; r += at_once) sum += hist[(t0 + r) * K + k];
+    atomicAdd(&s_sum[k], sum);
+  }
+  __syncthreads();
+  if (threadIdx.x < K) offsets[t0 * K + threadIdx.x] = s_sum[threadIdx.x];
+}
+
+// Block k: the chunks' sums to their starts, 1,024 chunks a step.
+constexpr int kStartThreads = 1024;
+
+__global__ void __launch_bounds__(kStartThreads) hash_chunk_starts_kernel(uint64_t n_chunks, int K, uint64_t *offsets) {
+  __shared__ unsigned long long s_warp[kStartThreads / 32];
   const int k = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint64_t t0 = blockIdx.y * kScanChunk, t = t0 + (uint64_t)kScanVec * threadIdx.x;
-  uint32_t mine[kScanVec], sum = 0;  // a tile counts at most 16,384: a chunk's sum fits 32 bits
+  unsigned long long before = 0;  // the sum of the steps before
+  for (uint64_t c0 = 0; c0 < n_chunks; c0 += kStartThreads) {
+    const uint64_t c = c0 + threadIdx.x;
+    uint64_t *const at = offsets + c * kScanChunk * K + k;
+    const unsigned long long mine = c < n_chunks ? *at : 0ull;
+    unsigned long long upto = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const unsigned long long o = __shfl_up_sync(0xffffffffu, upto, d);
+      if (lane >= d) upto += o;
+    }
+    if (lane == 31) s_warp[warp] = upto;
+    __syncthreads();
+    unsigned long long all = 0;
+    for (int w = 0; w < kStartThreads / 32; ++w) {
+      if (w == warp) upto += all;
+      all += s_warp[w];
+    }
+    if (c < n_chunks) *at = before + upto - mine;
+    before += all;
+    __syncthreads();  // before the next step's sums
+  }
+}
+
+// Block c K + k: chunk c of bucket k.
+__global__ void __launch_bounds__(kScanThreads) hash_scan_kernel(const uint32_t *hist, uint64_t n_htiles, int K,
+                                                                 bool has_starts, uint64_t *offsets) {
+  __shared__ unsigned long long s_before[kScanThreads / 32];
+  __shared__ uint32_t s_warp[kScanThreads / 32];
+  const uint32_t chunk = blockIdx.x / K, k = blockIdx.x % K;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint64_t t0 = chunk * kScanChunk, t = t0 + (uint64_t)kScanVec * threadIdx.x;
+  uint32_t mine[kScanVec], sum = 0;
 #pragma unroll
   for (int i = 0; i < kScanVec; ++i) sum += mine[i] = t + i < n_htiles ? hist[(t + i) * K + k] : 0u;
   unsigned long long before = 0;
+  if (has_starts) {
+    if (threadIdx.x == 0) before = offsets[t0 * K + k];
+  } else {
 #pragma unroll 8
-  for (uint64_t p = threadIdx.x; p < t0; p += 1024) before += hist[p * K + k];
+    for (uint64_t p = threadIdx.x; p < t0; p += kScanThreads) before += hist[p * K + k];
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(0xffffffffu, before, d);
+    for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(0xffffffffu, before, d);
+  }
   const uint32_t upto = warp_scan(sum);
   if (lane == 31) s_warp[warp] = upto;
   if (lane == 0) s_before[warp] = before;
-  __syncthreads();
+  __syncthreads();  // the start has been read as well
   unsigned long long at = __reduce_add_sync(0xffffffffu, lane < warp ? s_warp[lane] : 0u) + upto - sum;
-  for (int w = 0; w < 32; ++w) at += s_before[w];
+#pragma unroll
+  for (int w = 0; w < kScanThreads / 32; ++w) at += s_before[w];
 #pragma unroll
   for (int i = 0; i < kScanVec; ++i) {
     if (t + i < n_htiles) offsets[(t + i) * K + k] = at;
@@ -330,9 +392,13 @@ cudaError_t launch_hash_hist(const HashTensor *tensors, int n_tensors, uint64_t 
 cudaError_t launch_hash_scan(const uint32_t *hist, uint64_t n_htiles, int K, uint64_t *offsets,
                              cudaStream_t s) {
   if (n_htiles == 0) return cudaSuccess;
-  const uint64_t chunks = (n_htiles + kScanChunk - 1) / kScanChunk;
-  if (chunks > 65535) return cudaErrorInvalidValue;  // 4.4e12 elements
-  hash_scan_kernel<<<dim3(K, (unsigned)chunks), 1024, 0, s>>>(hist, n_htiles, K, offsets);
+  const uint64_t chunks = (n_htiles + kScanChunk - 1) / kScanChunk;  // chunks K < 2^27: n_htiles < 2^31
+  const bool starts = chunks > kScanReread;
+  if (starts) {
+    hash_chunk_sums_kernel<<<(unsigned)chunks, kSumThreads, 0, s>>>(hist, n_htiles, K, offsets);
+    hash_chunk_starts_kernel<<<K, kStartThreads, 0, s>>>(chunks, K, offsets);
+  }
+  hash_scan_kernel<<<(unsigned)(chunks * K), kScanThreads, 0, s>>>(hist, n_htiles, K, starts, offsets);
   return cudaGetLastError();
 }
 

@@ -30,3 +30,16 @@ def test_many_tensors(n_tensors):
         want = oracle.hash_list(numel, range(n_tensors), 4, 7, k)
         assert np.array_equal(subs[k].tensor.cpu().numpy(), want), k
     copes.check()
+
+
+@pytest.mark.parametrize("n_tensors", [1024, 1025, 12 * 1024, 12 * 1024 + 1, 1025 * 1024 + 5])
+def test_many_hash_tiles(n_tensors):
+    """A tensor takes a hash tile at least: one chunk of the scan over the tiles, several, and
+    more than the scan over the chunks takes in a step."""
+    from paper_2608_02391_gb300 import copes
+    K, numel = 3, np.ones(n_tensors, np.int64)
+    subs = copes.hash_partition(copes.Layout(numel), K, 7)
+    for k in range(K):
+        want = oracle.hash_list(numel, range(n_tensors), K, 7, k)
+        assert np.array_equal(subs[k].tensor.cpu().numpy(), want), k
+    copes.check()
