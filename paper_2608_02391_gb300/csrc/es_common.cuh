@@ -347,13 +347,28 @@ __device__ __forceinline__ GatherSmem gather_prologue(const UpdateArgs &a, char 
   return GatherSmem{row, WideTable(tab), a.n_alloc > (1ull << 34)};
 }
 
-// Element g's word of noise vector j, for any counter.
-static __device__ __noinline__ uint32_t gather_word_high(uint64_t g, uint32_t k0, uint32_t k1) {
-  uint32_t x[4];
-  const uint64_t q = g >> 2;
-  philox4x32_10((uint32_t)q, (uint32_t)(q >> 32), 0u, COPES_TAG_NOISE, k0, k1, x);
-  const uint32_t sel = (uint32_t)g & 3u;
-  return sel == 0 ? x[0] : (sel == 1 ? x[1] : (sel == 2 ? x[2] : x[3]));
+// sum_j w_j eps_j[g] for any counter (q, q_hi): q_hi only enters the folded keys u[2] and u[3]
+// (philox_folded_keys), which are formed here for each element.  Out of line, so that it takes
+// no registers from the form for counters below 2^32.
+static __device__ __noinline__ float gather_noise_sum_high(const UpdateArgs &a, const GatherSmem &s, uint64_t g) {
+  const uint64_t m = (uint64_t)kPhiloxM0 * (uint32_t)(g >> 2);
+  const bool h = (uint32_t)g & 2u, odd = (uint32_t)g & 1u;
+  float acc = 0.0f;
+  for (int j = 0; j < a.n_noise; ++j) {
+    uint32_t k[16];
+#pragma unroll
+    for (int r = 0; r < 16; r += 4) {
+      const uint4 v = *reinterpret_cast<const uint4 *>(&s.row[j][r]);
+      k[r] = v.x, k[r + 1] = v.y, k[r + 2] = v.z, k[r + 3] = v.w;
+    }
+    const uint64_t mk = (uint64_t)kPhiloxM0 * (a.seed_lo[j] ^ (uint32_t)(g >> 34));
+    k[2] = (uint32_t)(mk >> 32) ^ (a.seed_hi[j] + kPhiloxW1);     // round key 3
+    k[3] = (uint32_t)mk ^ (a.seed_hi[j] + 2u * kPhiloxW1);        // round key 5
+    const uint2 last = *reinterpret_cast<const uint2 *>(&s.row[j][h ? 18 : 16]);
+    const uint32_t wd = philox4x32_10_word((uint32_t)m, (uint32_t)(m >> 32), k, h, odd, last.x, last.y);
+    acc = __fmaf_rn(__uint_as_float(k[15]), normal_from_word(wd, s.tab), acc);
+  }
+  return acc;
 }
 
 // acc[u] = sum_j w_j eps_j[g[u]] (j ascending, one fp32 fma a term) for a thread's U elements.
@@ -364,6 +379,11 @@ template <int U, typename Index>
 __device__ __forceinline__ void gather_noise_sum(const UpdateArgs &a, const GatherSmem &s, const Index (&g)[U],
                                                  float (&acc)[U]) {
   static_assert(U % 2 == 0, "normals are paired");
+  if (s.high) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) acc[u] = gather_noise_sum_high(a, s, (uint64_t)g[u]);
+    return;
+  }
   uint32_t m0_lo[U], m0_hi[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
@@ -386,9 +406,6 @@ __device__ __forceinline__ void gather_noise_sum(const UpdateArgs &a, const Gath
       const uint2 last = *reinterpret_cast<const uint2 *>(&s.row[j][h ? 18 : 16]);
       wd[u] = philox4x32_10_word(m0_lo[u], m0_hi[u], k, h, odd, last.x, last.y);
     }
-    if (s.high)
-#pragma unroll
-      for (int u = 0; u < U; ++u) wd[u] = gather_word_high((uint64_t)g[u], a.seed_lo[j], a.seed_hi[j]);
     const float wj = __uint_as_float(k[15]);
 #pragma unroll
     for (int u = 0; u < U; u += 2) {  // two normals as one packed pair (bit-identical to one at a time)

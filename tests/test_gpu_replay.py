@@ -237,6 +237,40 @@ def test_hashing_past_counter_2_32_equals_the_mask(copes):
     copes.check()
 
 
+def test_updates_past_counter_2_32_equal_the_tiles(copes):
+    """Index-list and replayed updates on both sides of index 2^34, element for element those
+    over TILES (checked against the oracle there)."""
+    lo, n = 1 << 34, (1 << 34) + 70_001
+    first = lo - 70_000
+    a = copes.Arena(torch.zeros(n, dtype=torch.bfloat16, device="cuda"), torch.zeros(n, device="cuda"))
+    theta = torch.randn(n - first, device="cuda")
+    nid, sign, P = copes.member_table(6, copes.ANTITHETIC)
+    f = torch.linspace(-1, 1, 6, device="cuda")
+
+    def update(sub):
+        a.master[first:] = theta
+        a.w[first:] = 0
+        copes.update(a, sub, nid, sign, f, copes.member_seeds(33, 1, 2, P), 1e-2)
+        return a.master[first:].clone(), a.w[first:].clone()
+
+    want = update(copes.tiles_from_ranges([(first, n)]))
+    assert (want[0] != theta).sum() > 0.99 * theta.numel()
+    index = torch.arange(first, n, device="cuda")
+    got = update(copes.SubspaceHandle(copes.SUBSPACE_INDICES, index, index.numel()))
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    sub = copes.hash_replay_partition(copes.Layout([lo, n - lo]), 16, 77, count=False)[3]
+    for masked in (False, True):
+        if masked:
+            copes.hash_replay_mask(a, sub)
+        got = update(sub)
+        member = got[0] != theta
+        for side in (member[:lo - first], member[lo - first:]):
+            assert 0.8 * side.numel() < 16 * side.sum() < 1.2 * side.numel()
+        assert torch.equal(got[0][member], want[0][member]) and torch.equal(got[1][member], want[1][member])
+        assert not got[1][~member].any()
+    copes.check()
+
+
 @pytest.mark.parametrize("tiles", [1, 5, 607, 1216, 1300, 1830, 2433])
 def test_any_number_of_hash_tiles_equals_the_lists(copes, tiles):
     """The kernels' blocks take 1 to 4 consecutive hash tiles, by the number of tiles."""
