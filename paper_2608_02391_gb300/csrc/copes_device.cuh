@@ -83,8 +83,9 @@ struct NormalTable {
   uint32_t base;
 
   // Fills a block's table (every load in flight before the first store); a __syncthreads
-  // must follow before the constructor.
-  static __device__ __forceinline__ void fill(float4 *s_tab) {
+  // must follow before the constructor.  `between` runs after the loads have been asked for.
+  template <typename Between>
+  static __device__ __forceinline__ void fill(float4 *s_tab, Between between) {
     constexpr int kSteps = (kFloat4s + kThreads - 1) / kThreads;
     float4 v[kSteps];
 #pragma unroll
@@ -92,11 +93,15 @@ struct NormalTable {
       const int i = threadIdx.x + k * kThreads;
       if (i < kFloat4s) v[k] = g_normal_table[i / C];
     }
+    between();
 #pragma unroll
     for (int k = 0; k < kSteps; ++k) {
       const int i = threadIdx.x + k * kThreads;
       if (i < kFloat4s) s_tab[i] = v[k];
     }
+  }
+  static __device__ __forceinline__ void fill(float4 *s_tab) {
+    fill(s_tab, [] {});
   }
 
   // This lane's view of the table, after the fill's barrier: entry i is at base + (f << kShift)

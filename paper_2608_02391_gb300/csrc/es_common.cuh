@@ -257,12 +257,14 @@ __device__ __forceinline__ UpdateSmem update_prologue(const UpdateArgs &a, char 
   float4 *tab = reinterpret_cast<float4 *>(smem);
   uint32_t(*fk)[20] = reinterpret_cast<uint32_t (*)[20]>(smem + kUpdateSmemBytes);
   float2 *w = reinterpret_cast<float2 *>(smem + kUpdateSmemBytes + a.n_noise * 80);
-  WideTable::fill(tab);
-  noise_keys_to_smem(a, 0, fk);
-  for (int j = threadIdx.x; j < a.n_noise; j += blockDim.x) {
-    const float wj = noise_weight(a, j);
-    w[j] = make_float2(wj, wj);
-  }
+  // the last warps fold the members, the first the keys, while the table is on its way
+  WideTable::fill(tab, [&] {
+    for (int j = kThreads - 1 - threadIdx.x; j < a.n_noise; j += blockDim.x) {
+      const float wj = noise_weight(a, j);
+      w[j] = make_float2(wj, wj);
+    }
+    noise_keys_to_smem(a, 0, fk);
+  });
   __syncthreads();
   return UpdateSmem{fk, w, WideTable(tab), 0};
 }
