@@ -212,10 +212,6 @@ __device__ __forceinline__ void elem_range(const ElemArgs &a, const WideTable &t
                                            NextUnit &next) {
   constexpr uint32_t kStep = 4u * kThreads * G;
   uint32_t at = 0;
-    if (has_edge) {
-      WStore<WT>::one(a.w, edge, edge_v);
-      store_copies_one<WT>(a.copies, edge, edge_v);
-    }
   for (; at + kStep / 2 < n; at += kStep) {
     if (at + kStep + kStep / 2 >= n) next.ask();
     elem_step<OP, WT, G, true, true>(a, tab, b, at + 4u * threadIdx.x, n);
@@ -345,6 +341,10 @@ __global__ void __launch_bounds__(kThreads, 3) restore_tiles_kernel(const __grid
         WStore<WT>::full(a.w, lo + o, v);
         store_copies_full<WT>(a.copies, lo + o, v);
       }
+    }
+    if (has_edge) {
+      WStore<WT>::one(a.w, edge, edge_v);
+      store_copies_one<WT>(a.copies, edge, edge_v);
     }
   });
 }
