@@ -108,20 +108,25 @@ __device__ __forceinline__ uint32_t warp_scan(uint32_t v) {
   return v;
 }
 
-// The exclusive prefix sums of hist[tile][k] over the tiles, per bucket k, in chunks of 1,024
-// tiles.  Up to kScanReread chunks, a chunk's block sums the tiles before it itself; beyond,
-// two launches before it are linear in the tiles: the sums of the chunks, and their scan.
-// Until the last launch, the start of a chunk lies in offsets at the chunk's first tile,
-// which is where it belongs.  Re-read / with the launches before, us: 8,545 tiles, K = 16 and 64
-// 6.0 / 10.7 and 17 / 24; 12,208 tiles 10.2 / 12.3 and 28 / 26; 30,518 tiles 29 / 15 and 122 / 36;
-// 488,282 tiles 3,209 / 88 and 27,858 / 353.
-constexpr int kScanVec = 4;  // consecutive tiles a thread
-constexpr int kScanThreads = 256;
+// The exclusive prefix sums of hist[tile][k] over the tiles, per bucket k, in chunks of tiles.  A
+// chunk's block sums the tiles before it itself while that is little (hash_scan_rereads);
+// beyond, two launches before it are linear in the tiles: the sums of the chunks, and their
+// scan.  Until the last launch, the start of a chunk lies in offsets at the chunk's first
+// tile, which is where it belongs.
+constexpr int kScanVec = 4;         // consecutive tiles a thread
+constexpr int kScanThreads = 256;   // with starts
+constexpr int kRereadThreads = 1024;
 constexpr uint64_t kScanChunk = kScanVec * kScanThreads;
-constexpr uint64_t kScanReread = 12;
 constexpr int kSumThreads = 1024;
-static_assert(kScanChunk * kHashTile < 1ull << 32, "a chunk's sum fits 32 bits");
+static_assert((uint64_t)kScanVec * kRereadThreads * kHashTile < 1ull << 32, "a chunk's sum fits 32 bits");
 static_assert(COPES_MAX_K <= kSumThreads, "a thread per bucket");
+
+// Re-read / with the launches before, us: 12,208 tiles, K = 16 and 64 9.3 / 12.3 and 21 / 26; 30,518
+// tiles 13.8 / 14.9 and 58 / 36; 488,282 tiles 915 / 88 and 6,393 / 353; and two launches more.
+static bool hash_scan_rereads(uint64_t n_htiles, int K) {
+  const uint64_t chunks = (n_htiles + kScanVec * kRereadThreads - 1) / (kScanVec * kRereadThreads);
+  return chunks <= 40 && chunks * chunks * (uint64_t)K <= 1600;
+}
 
 __global__ void __launch_bounds__(kSumThreads) hash_chunk_sums_kernel(const uint32_t *hist, uint64_t n_htiles, int K,
                                                                        uint64_t *offsets) {
@@ -170,25 +175,26 @@ __global__ void __launch_bounds__(kStartThreads) hash_chunk_starts_kernel(uint64
   }
 }
 
-// Block c K + k: chunk c of bucket k.
-__global__ void __launch_bounds__(kScanThreads) hash_scan_kernel(const uint32_t *hist, uint64_t n_htiles, int K,
-                                                                 bool has_starts, uint64_t *offsets) {
-  __shared__ unsigned long long s_before[kScanThreads / 32];
-  __shared__ uint32_t s_warp[kScanThreads / 32];
+// Block c K + k: chunk c, of kScanVec THREADS tiles, of bucket k.
+template <int THREADS, bool REREAD>
+__global__ void __launch_bounds__(THREADS) hash_scan_kernel(const uint32_t *hist, uint64_t n_htiles, int K,
+                                                            uint64_t *offsets) {
+  __shared__ unsigned long long s_before[THREADS / 32];
+  __shared__ uint32_t s_warp[THREADS / 32];
   const uint32_t chunk = blockIdx.x / K, k = blockIdx.x % K;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint64_t t0 = chunk * kScanChunk, t = t0 + (uint64_t)kScanVec * threadIdx.x;
+  const uint64_t t0 = chunk * (uint64_t)(kScanVec * THREADS), t = t0 + (uint64_t)kScanVec * threadIdx.x;
   uint32_t mine[kScanVec], sum = 0;
 #pragma unroll
   for (int i = 0; i < kScanVec; ++i) sum += mine[i] = t + i < n_htiles ? hist[(t + i) * K + k] : 0u;
   unsigned long long before = 0;
-  if (has_starts) {
-    if (threadIdx.x == 0) before = offsets[t0 * K + k];
-  } else {
+  if (REREAD) {
 #pragma unroll 8
-    for (uint64_t p = threadIdx.x; p < t0; p += kScanThreads) before += hist[p * K + k];
+    for (uint64_t p = threadIdx.x; p < t0; p += THREADS) before += hist[p * K + k];
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(0xffffffffu, before, d);
+  } else if (threadIdx.x == 0) {
+    before = offsets[t0 * K + k];
   }
   const uint32_t upto = warp_scan(sum);
   if (lane == 31) s_warp[warp] = upto;
@@ -196,7 +202,7 @@ __global__ void __launch_bounds__(kScanThreads) hash_scan_kernel(const uint32_t 
   __syncthreads();  // the start has been read as well
   unsigned long long at = __reduce_add_sync(0xffffffffu, lane < warp ? s_warp[lane] : 0u) + upto - sum;
 #pragma unroll
-  for (int w = 0; w < kScanThreads / 32; ++w) at += s_before[w];
+  for (int w = 0; w < THREADS / 32; ++w) at += s_before[w];
 #pragma unroll
   for (int i = 0; i < kScanVec; ++i) {
     if (t + i < n_htiles) offsets[(t + i) * K + k] = at;
@@ -392,13 +398,16 @@ cudaError_t launch_hash_hist(const HashTensor *tensors, int n_tensors, uint64_t 
 cudaError_t launch_hash_scan(const uint32_t *hist, uint64_t n_htiles, int K, uint64_t *offsets,
                              cudaStream_t s) {
   if (n_htiles == 0) return cudaSuccess;
-  const uint64_t chunks = (n_htiles + kScanChunk - 1) / kScanChunk;  // chunks K < 2^27: n_htiles < 2^31
-  const bool starts = chunks > kScanReread;
-  if (starts) {
+  if (hash_scan_rereads(n_htiles, K)) {
+    constexpr uint64_t kChunk = kScanVec * kRereadThreads;
+    const unsigned blocks = (unsigned)((n_htiles + kChunk - 1) / kChunk * K);
+    hash_scan_kernel<kRereadThreads, true><<<blocks, kRereadThreads, 0, s>>>(hist, n_htiles, K, offsets);
+  } else {
+    const uint64_t chunks = (n_htiles + kScanChunk - 1) / kScanChunk;  // chunks K <= 2^27: n_htiles < 2^31
     hash_chunk_sums_kernel<<<(unsigned)chunks, kSumThreads, 0, s>>>(hist, n_htiles, K, offsets);
     hash_chunk_starts_kernel<<<K, kStartThreads, 0, s>>>(chunks, K, offsets);
+    hash_scan_kernel<kScanThreads, false><<<(unsigned)(chunks * K), kScanThreads, 0, s>>>(hist, n_htiles, K, offsets);
   }
-  hash_scan_kernel<<<(unsigned)(chunks * K), kScanThreads, 0, s>>>(hist, n_htiles, K, starts, offsets);
   return cudaGetLastError();
 }
 

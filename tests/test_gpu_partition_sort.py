@@ -32,12 +32,13 @@ def test_many_tensors(n_tensors):
     copes.check()
 
 
-@pytest.mark.parametrize("n_tensors", [1024, 1025, 12 * 1024, 12 * 1024 + 1, 1025 * 1024 + 5])
-def test_many_hash_tiles(n_tensors):
-    """A tensor takes a hash tile at least: one chunk of the scan over the tiles, several, and
-    more than the scan over the chunks takes in a step."""
+@pytest.mark.parametrize("n_tensors,K", [(4096, 3), (4097, 3), (8 * 4096, 16), (8 * 4096 + 1, 16), (24 * 4096, 3),
+                                         (12_289, 64), (20_481, 64), (1025 * 1024 + 5, 3)])
+def test_many_hash_tiles(n_tensors, K):
+    """A tensor takes a hash tile at least: one chunk of the scan over the tiles, several, on both
+    sides of where chunks are summed first, and more than their scan takes in a step."""
     from paper_2608_02391_gb300 import copes
-    K, numel = 3, np.ones(n_tensors, np.int64)
+    numel = np.ones(n_tensors, np.int64)
     subs = copes.hash_partition(copes.Layout(numel), K, 7)
     for k in range(K):
         want = oracle.hash_list(numel, range(n_tensors), K, 7, k)
