@@ -119,7 +119,7 @@ typedef struct {
   const uint64_t *tiles;   /* TILES: device [2 * n_tiles]                                */
   uint64_t n_tiles;
   const int64_t *index;    /* INDICES: device [n_index]                                  */
-  uint64_t n_index;
+  uint64_t n_index;        /* INDICES: entries of the list; TILES: optional COPES_TILES_HINT */
   const void *replay;      /* HASH_REPLAY: device tensor table (copes_hash_replay_subspace) */
   uint64_t n_replay_tiles; /* HASH_REPLAY: 16,384-element hash tiles the table covers     */
   int n_replay_tensors;    /* HASH_REPLAY: entries of the table                           */
@@ -131,6 +131,12 @@ typedef struct {
   uint32_t *replay_mask;   /* HASH_REPLAY, optional: device membership bits filled by
                               copes_hash_replay_mask; NULL: membership is hashed */
 } copes_subspace;
+
+/* TILES: what a caller may say of the tiles in n_index (0: nothing): the elements of all of them
+ * and whether they all begin at multiples of 4.  Launches are cut by it: it changes how long
+ * they take (tiles of unusual length or place several times longer without it), never a
+ * result. */
+#define COPES_TILES_HINT(elements, aligned) (((uint64_t)(elements) << 1) | ((aligned) ? 1u : 0u))
 
 /* Parameter layout: the model's tensors in order. */
 typedef struct {

@@ -266,13 +266,14 @@ class SubspaceHandle:
     replay: Optional[Subspace] = None
     gathered: Optional[torch.Tensor] = None  # INDICES: theta in list order (gather_master)
     mask: Optional[torch.Tensor] = None      # HASH_REPLAY: membership bits (hash_replay_mask)
+    aligned: bool = True                     # TILES: whether every tile begins at a multiple of 4 (speed only)
 
     def struct(self) -> Subspace:
         if self.kind == SUBSPACE_HASH_REPLAY:
             return self.replay
         if self.kind == SUBSPACE_TILES:
             return Subspace(SUBSPACE_TILES, self.tensor.data_ptr() if self.tensor.numel() else None,
-                            self.tensor.shape[0], None, 0)
+                            self.tensor.shape[0], None, max(self.numel, 0) << 1 | self.aligned)
         S = Subspace(SUBSPACE_INDICES, None, 0, self.tensor.data_ptr() if self.tensor.numel() else None,
                      self.tensor.numel())
         if self.gathered is not None:
@@ -280,7 +281,7 @@ class SubspaceHandle:
         return S
 
 
-def _tiles_result(count_fn, fill_fn, device, stream) -> SubspaceHandle:
+def _tiles_result(count_fn, fill_fn, aligned: bool, device, stream) -> SubspaceHandle:
     count = ctypes.c_uint64(0)
     _check(count_fn(ctypes.byref(count)))
     n = int(count.value)
@@ -288,7 +289,7 @@ def _tiles_result(count_fn, fill_fn, device, stream) -> SubspaceHandle:
     _check(fill_fn(tiles, n, ctypes.byref(count)))
     t = tiles[:n]
     numel = int((t[:, 1] - t[:, 0]).sum().item()) if n else 0
-    return SubspaceHandle(SUBSPACE_TILES, t, numel)
+    return SubspaceHandle(SUBSPACE_TILES, t, numel, aligned=aligned)
 
 
 def tiles_from_ranges(ranges, tile_size: int = DEFAULT_TILE, device="cuda", stream=None) -> SubspaceHandle:
@@ -298,7 +299,8 @@ def tiles_from_ranges(ranges, tile_size: int = DEFAULT_TILE, device="cuda", stre
     return _tiles_result(
         lambda cnt: L.copes_tiles_from_ranges(_np_ptr(b), _np_ptr(e), len(ranges), tile_size, None, 0, cnt, s),
         lambda t, n, cnt: L.copes_tiles_from_ranges(_np_ptr(b), _np_ptr(e), len(ranges), tile_size,
-                                                    _ptr(t), n, cnt, s), device, stream)
+                                                    _ptr(t), n, cnt, s),
+        tile_size % 4 == 0 and not (b & np.uint64(3)).any(), device, stream)
 
 
 def subspace_build(layout: Layout, mode: int, K: int, k: int, seed: int = 0, chunk: int = 65536,
@@ -309,11 +311,19 @@ def subspace_build(layout: Layout, mode: int, K: int, k: int, seed: int = 0, chu
     spec = PartitionSpec(mode, K, seed, chunk, _np_ptr(g))
     L, s = load(), _stream(stream)
     cm = _ptr(chunk_map)
+    # tensors begin at multiples of 64, chunks too: only a contiguous subspace may begin elsewhere
+    first = 0
+    if mode == PART_CONTIGUOUS and 0 <= k < K:
+        upto = np.cumsum(layout.numel)
+        lo = int(upto[-1]) * k // K
+        t = int(np.searchsorted(upto, np.uint64(lo), side="right"))
+        first = lo - int(upto[t - 1]) if t else lo  # into its tensor
     return _tiles_result(
         lambda cnt: L.copes_subspace_build(ctypes.byref(layout.desc), ctypes.byref(spec), k, tile_size,
                                            cm, None, 0, cnt, s),
         lambda t, n, cnt: L.copes_subspace_build(ctypes.byref(layout.desc), ctypes.byref(spec), k,
-                                                 tile_size, cm, _ptr(t), n, cnt, s), device, stream)
+                                                 tile_size, cm, _ptr(t), n, cnt, s),
+        tile_size % 4 == 0 and first % 4 == 0, device, stream)
 
 
 def random_chunk_map(n_chunks: int, K: int, seed: int, device="cuda", stream=None) -> torch.Tensor:

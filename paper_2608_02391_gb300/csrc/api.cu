@@ -17,39 +17,6 @@
 using copes::ElemArgs;
 using copes::UpdateArgs;
 
-// Few tiles would leave SMs without work, or the last of two or three waves of blocks nearly
-// empty: they are cut into parts.  Short tiles are joined into runs of about 16,384 elements
-// instead, while enough units are left.  Only a bound of the mean tile length is known
-// here (disjoint tiles: n_alloc / n_tiles), so no part is made shorter than 1,024 elements
-// by that bound; a part of a tile that turns out shorter may come out empty.
-// Measured (bf16, 16,384-element tiles; one block a tile / one unit a tile / these parts): the
-// two-pairs perturb of 2^18, 2^20 and 14.9M elements 7.6 / 7.5 / 3.3, 8.0 / 7.8 / 4.5 and
-// 39.2 / 36.5 / 34.1 us; tiles of 1,000 elements joined, 11.1M elements: perturb 29.0 -> 18.8
-// us, update (P = 16) 351 -> 176.  The update brings its own cut (log_parts).
-// The bound is loose by as much as the subspace is a part of the arena, and a run then holds
-// less than it says: short tiles are joined while 500 units are left, and those of a middling
-// bound up to 32,768 elements by it while there are eight waves of units.  Tiles of 1,000 in a
-// third of the arena, 4, 11.1 and 134M elements, only eight waves of at most 16,384 / these:
-// perturb 17.0 / 10.4, 30.6 / 20.7 and 205 / 172 us, update (P = 7) 38.2 / 36.2, 92.9 / 86.4 and
-// 919 / 881.  From 3,500 on whole tiles are long enough (aligned tiles of 4,096, 11.1M
-// elements: pair 17.2 / 19.8).
-copes::TileUnits copes::plan_tile_units(uint64_t n_tiles, uint64_t n_alloc, uint32_t log_parts, uint32_t few) {
-  TileUnits u{(uint32_t)n_tiles, 0, 1};
-  const uint64_t bound = std::max<uint64_t>(1, n_alloc / n_tiles);  // >= the mean tile length
-  if (bound > 8192) {
-    if (n_tiles < few && n_tiles < 1u << 24) u.log_parts = log_parts;  // the grid stays in 32 bits
-  } else if (n_tiles < 500) {
-    while ((n_tiles << (u.log_parts + 1)) <= 500 && (bound >> (u.log_parts + 1)) >= 1024) ++u.log_parts;
-  } else {
-    auto run = [&](uint64_t elements, uint64_t left) { return std::min(elements / bound, n_tiles / left); };
-    const uint64_t eight_waves = run(bound < 2048 || bound >= 3500 ? 16384 : 32768, 8 * 608);
-    const uint64_t r = bound < 3500 ? std::max(run(16384, 500), eight_waves) : eight_waves;
-    u.run = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(r, 1), 32);
-  }
-  u.n_units = (uint32_t)(u.run > 1 ? (n_tiles + u.run - 1) / u.run : n_tiles << u.log_parts);
-  return u;
-}
-
 namespace {
 
 thread_local std::string g_message;
@@ -216,6 +183,7 @@ ElemArgs elem_args(const copes_params *p, const copes_subspace *S) {
   if (S->kind == COPES_SUBSPACE_TILES) {
     a.tiles = S->tiles;
     a.n_tiles = S->n_tiles;
+    a.tile_hint = S->n_index;
   } else {
     a.index = S->index;
     a.n_index = S->n_index;
@@ -320,7 +288,8 @@ int copes_last_error(char *buf, size_t len) {
 int copes_check(cudaStream_t stream) {
   cudaError_t e = cudaStreamSynchronize(stream);
   if (e != cudaSuccess) return cuda_fail(e, "copes_check");
-  const unsigned bits = copes::read_and_clear_es_errors() | copes::read_and_clear_partition_errors() |
+  const unsigned bits = copes::read_and_clear_es_errors() | copes::read_and_clear_ragged_errors() |
+                        copes::read_and_clear_partition_errors() |
                         copes::read_and_clear_replay_errors() | copes::read_and_clear_backup_errors();
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "copes_check");
   if (bits)
@@ -798,6 +767,7 @@ int run_backup_elementwise(int op, const copes_backup_params *p, const copes_sub
   a.n_alloc = p->n_alloc;
   a.tiles = S->tiles;
   a.n_tiles = S->n_tiles;
+  a.tile_hint = S->n_index;
   a.seed_lo = (uint32_t)seed;
   a.seed_hi = (uint32_t)(seed >> 32);
   a.a = sigma;
@@ -824,6 +794,7 @@ int copes_update(const copes_params *p, const copes_subspace *S, int n_members,
   if (S->kind == COPES_SUBSPACE_TILES) {
     a.tiles = S->tiles;
     a.n_tiles = S->n_tiles;
+    a.tile_hint = S->n_index;
   } else {
     a.index = S->index;
     a.n_index = S->n_index;
@@ -868,6 +839,7 @@ int copes_backup_perturb_partner(const copes_backup_params *p, const copes_subsp
   a.n_alloc = p->n_alloc;
   a.tiles = S->tiles;
   a.n_tiles = S->n_tiles;
+  a.tile_hint = S->n_index;
   a.partner = const_cast<void *>(partner);
   a.partner_base = partner_base;
   a.partner_len = partner_len;
@@ -892,6 +864,7 @@ int copes_backup_update(const copes_backup_params *p, const copes_subspace *S, i
   a.n_alloc = p->n_alloc;
   a.tiles = S->tiles;
   a.n_tiles = S->n_tiles;
+  a.tile_hint = S->n_index;
   return launch_status(copes::launch_backup_update(a, dev, stream), who);
 }
 

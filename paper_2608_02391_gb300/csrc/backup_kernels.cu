@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kThreads, kBackupUpdateBlocksPerSM)
 
 cudaError_t launch_backup_elementwise(int op, ElemArgs &a, uint16_t *backup, cudaStream_t s) {
   if (a.n_tiles == 0) return cudaSuccess;
-  a.units = plan_tile_units(a.n_tiles, a.n_alloc, 2, 1216);
+  a.units = plan_backup(tile_work(a.n_tiles, a.n_alloc, a.tile_hint), 4096);
   const unsigned grid = a.units.n_units;
   switch (op) {
     case kBackupSave: backup_elem_kernel<kBackupSave><<<grid, kThreads, 0, s>>>(a, backup); break;
@@ -172,7 +172,8 @@ cudaError_t launch_backup_elementwise(int op, ElemArgs &a, uint16_t *backup, cud
 cudaError_t launch_backup_update(UpdateArgs &a, uint16_t *backup, cudaStream_t s) {
   if (a.n_tiles == 0) return cudaSuccess;
   // eighths up to two waves of whole tiles: 11.1M elements (P = 8) 184 us whole, 142 in eighths
-  a.units = plan_tile_units(a.n_tiles, a.n_alloc, 3, 8 * 152 + 1);
+  // eighths up to two waves of whole tiles: 11.1M elements (P = 8) 184 us whole, 142 in eighths
+  a.units = plan_backup(tile_work(a.n_tiles, a.n_alloc, a.tile_hint), 2048);
   backup_update_kernel<<<a.units.n_units, kThreads, update_smem_bytes(a.n_noise), s>>>(a, backup);
   return cudaGetLastError();
 }

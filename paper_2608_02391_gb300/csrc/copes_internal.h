@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "../../include/copes.h"
+#include "tile_units.h"
 
 namespace copes {
 
@@ -102,6 +103,19 @@ __host__ __device__ __forceinline__ void philox_folded_keys(const uint32_t rk[20
   u[19] = 0;
 }
 
+// The folded keys for another high word c1 (c2 = 0), from those for c1 = 0 and the round keys:
+// only u[2] and u[3] differ.
+struct HighKeys {
+  const uint32_t *u0;
+  uint32_t u2, u3;
+  __host__ __device__ __forceinline__ HighKeys(const uint32_t *folded, const uint32_t *rk, uint32_t c1) : u0(folded) {
+    const uint64_t mk = (uint64_t)kPhiloxM0 * (rk[0] ^ c1);
+    u2 = (uint32_t)(mk >> 32) ^ rk[3];
+    u3 = (uint32_t)mk ^ rk[5];
+  }
+  __host__ __device__ __forceinline__ uint32_t operator[](int i) const { return i == 2 ? u2 : (i == 3 ? u3 : u0[i]); }
+};
+
 template <typename U>
 __host__ __device__ __forceinline__ void philox4x32_10_folded(uint32_t m0_lo, uint32_t m0_hi, const U &u,
                                                               uint32_t out[4]) {
@@ -191,13 +205,6 @@ enum : unsigned {
 };
 
 // ---------------------------------------------------------------- launch arguments
-// How a launch over TILES is cut into units, one grid block each (plan_tile_units): with
-// g = u >> log_parts, unit u covers part u - (g << log_parts) of the tiles
-// [g run, (g + 1) run).
-struct TileUnits {
-  uint32_t n_units, log_parts, run;
-};
-
 // Whether [b, e), as read from a device tile table, is a tile of the arena.  The kernels touch
 // nothing of a tile before this has held: e - b alone says nothing of a tile with b > e,
 // where it wraps.
@@ -239,8 +246,9 @@ struct ElemArgs {
   WorkingCopies copies;  // restore / commit / init write these as well as w
   uint32_t rk_b[20];            // kOpPerturbTwoPairs: the second noise vector's round keys
   uint32_t fk[20], fk_b[20];    // folded keys (philox_folded_keys, tag) for counters below 2^32
-  TileUnits units;   // TILES
-  uint32_t segment;  // INDICES: list entries per block
+  uint64_t tile_hint;  // TILES: copes_subspace.n_index
+  TileUnits units;     // TILES
+  uint32_t segment;    // INDICES: list entries per block
 };
 
 // kOpGather / kOpScatter copy theta between master and the gathered copy (INDICES only).
@@ -280,6 +288,7 @@ struct UpdateArgs {
   int8_t sign[COPES_MAX_MEMBERS];
   float *gathered;  // INDICES: theta in list order instead of master[index[p]] (or NULL)
   WorkingCopies copies;  // the fused commit writes these as well as w
+  uint64_t tile_hint;    // TILES: copes_subspace.n_index
   TileUnits units;       // TILES
   uint32_t segment;      // INDICES: list entries per block
 };
@@ -295,12 +304,10 @@ inline cudaError_t allow_smem(const void *kernel, uint32_t total, uint32_t most)
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
-// The units of a launch over n_tiles disjoint tiles of an n_alloc-element arena (n_tiles in
-// [1, 2^31)): fewer tiles than `few` are cut into 2^log_parts parts each.
-TileUnits plan_tile_units(uint64_t n_tiles, uint64_t n_alloc, uint32_t log_parts, uint32_t few);
-
 // launch_elementwise and launch_update fill in a.units and a.segment.
 cudaError_t launch_elementwise(int op, int kind, int dtype, ElemArgs &a, cudaStream_t s);
+// The noise ops over tiles that are not default_like, or of an arena past 2^34 elements.
+cudaError_t launch_elem_ragged(int op, int dtype, const ElemArgs &a, cudaStream_t s);
 cudaError_t launch_update(int kind, int dtype, UpdateArgs &a, cudaStream_t s);
 cudaError_t launch_shape(const float *r, int n, const int32_t *group, int mode, float *f,
                          cudaStream_t s);
@@ -381,6 +388,7 @@ void set_last_error(const char *message);
 
 // Device error words of each translation unit: read and clear (synchronous).
 unsigned read_and_clear_es_errors();
+unsigned read_and_clear_ragged_errors();
 unsigned read_and_clear_partition_errors();
 unsigned read_and_clear_replay_errors();
 unsigned read_and_clear_backup_errors();

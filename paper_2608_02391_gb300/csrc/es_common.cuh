@@ -72,17 +72,16 @@ __device__ __forceinline__ bool unit_answer(const UnitSmem &s, uint32_t &unit) {
   return ok != 0;
 }
 
-// Part `part` of the elements [b, e): equal stretches of whole steps, cut at multiples of 4;
-// the last one takes what is left over.
+// Part `part` of the elements [b, e): as many steps as the others to within one, from the group of
+// b on; the three elements that a cut group may leave over are the last one's.
 __device__ __forceinline__ void tile_part(const TileUnits &u, uint32_t part, uint64_t &b, uint64_t &e) {
   constexpr uint32_t kStep = 4 * kThreads;
   const uint64_t lo = b & ~3ull;
-  const uint32_t part_len = (uint32_t)(e - lo) >> u.log_parts;  // of at most COPES_TILE_MAX + 3
-  const uint32_t chunk = max(kStep, (part_len + kStep / 2) / kStep * kStep);
-  const uint64_t p0 = lo + (uint64_t)part * chunk;
-  const bool last = part + 1 == (1u << u.log_parts);
+  const uint32_t steps = max(((uint32_t)(e - lo) + kStep - 4) / kStep, 1u);  // of at most COPES_TILE_MAX + 66
+  const uint64_t p0 = lo + (part * steps >> u.log_parts) * kStep;
+  const uint64_t p1 = lo + ((part + 1) * steps >> u.log_parts) * kStep;
   b = min(max(b, p0), e);
-  e = last ? e : max(b, min(e, p0 + chunk));
+  if (part + 1 != 1u << u.log_parts) e = max(b, min(e, p1));
 }
 
 // Runs body(b, e) for the stretches of one unit: the part of its tile, or its run of tiles with

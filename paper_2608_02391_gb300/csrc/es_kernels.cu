@@ -6,6 +6,7 @@
 
 #include "copes_device.cuh"
 #include "copes_internal.h"
+#include "elem_ops.cuh"
 #include "es_common.cuh"
 
 namespace copes {
@@ -15,120 +16,8 @@ __device__ unsigned int g_es_error = 0;
 __device__ __forceinline__ void flag_error(unsigned bit) { atomicOr(&g_es_error, bit); }
 
 // ------------------------------------------------------------ perturb / restore / init
-// A "group" is the 4 consecutive global indices 4q .. 4q+3, which share Philox counter q.
 template <int OP>
 constexpr uint32_t op_tag() { return OP == kOpInit ? COPES_TAG_INIT : COPES_TAG_NOISE; }
-
-// Ops whose values are the context (restore / commit, init) go to the other working copies
-// too; perturbations go to the buffers their call names.
-template <int OP>
-constexpr bool writes_context() { return OP == kOpRestore || OP == kOpInit; }
-
-// Noise vectors and values an op forms per element: the perturb theta + a eps, the pair also
-// theta - a eps, the two pairs theta +- a eps_A and theta +- a eps_B, init b + a eps.
-template <int OP>
-constexpr int op_noises() { return OP == kOpPerturbTwoPairs ? 2 : 1; }
-template <int OP>
-constexpr int op_values() { return OP == kOpPerturbTwoPairs ? 4 : (OP == kOpPerturbPair ? 2 : 1); }
-
-// The values of one group from its noise (e2[s]: noise vector s as packed pairs) and theta:
-// v[0] = fma(a, eps, theta), and with the antithetic sign v[1] = fma(-a, eps, theta) (pair;
-// the two pairs' v[2], v[3] from the second vector): each bit for bit what kOpPerturb
-// computes with that noise vector and sign.
-template <int OP>
-__device__ __forceinline__ void group_values(const ElemArgs &a, const unsigned long long (*e2)[2],
-                                             const float (&th)[4], float (&v)[op_values<OP>()][4]) {
-#pragma unroll
-  for (int p = 0; p < 2; ++p) {
-    const unsigned long long t2 = OP == kOpInit ? splat_f32x2(a.b) : pack_f32x2(th[2 * p], th[2 * p + 1]);
-#pragma unroll
-    for (int m = 0; m < op_values<OP>(); ++m)
-      unpack_f32x2(fma_f32x2(splat_f32x2((m & 1) ? -a.a : a.a), e2[m >> 1][p], t2), v[m][2 * p], v[m][2 * p + 1]);
-  }
-}
-
-// Value m of an op goes to w (m = 0), the partner buffer (the pair's m = 1) or the further
-// working copies (the two pairs' m = 1 .. 3); the context's only value to all copies.
-template <int OP, typename WT>
-__device__ __forceinline__ void store_values_full(const ElemArgs &a, uint64_t g, const float (&v)[op_values<OP>()][4]) {
-  if (OP == kOpInit) st_stream_f4(a.master + g, make_float4(v[0][0], v[0][1], v[0][2], v[0][3]));
-  WStore<WT>::full(a.w, g, v[0]);
-  if constexpr (writes_context<OP>()) store_copies_full<WT>(a.copies, g, v[0]);
-  if constexpr (OP == kOpPerturbPair) WStore<WT>::full(a.partner, g - a.partner_base, v[1]);
-  if constexpr (OP == kOpPerturbTwoPairs) {
-#pragma unroll
-    for (int m = 1; m < 4; ++m) WStore<WT>::full(a.copies.p[m - 1], g, v[m]);
-  }
-}
-
-template <int OP, typename WT>
-__device__ __forceinline__ void store_values_one(const ElemArgs &a, uint64_t g, const float (&v)[op_values<OP>()][4],
-                                                 int k) {
-  if (OP == kOpInit) a.master[g] = v[0][k];
-  WStore<WT>::one(a.w, g, v[0][k]);
-  if constexpr (writes_context<OP>()) store_copies_one<WT>(a.copies, g, v[0][k]);
-  if constexpr (OP == kOpPerturbPair) WStore<WT>::one(a.partner, g - a.partner_base, v[1][k]);
-  if constexpr (OP == kOpPerturbTwoPairs) {
-#pragma unroll
-    for (int m = 1; m < 4; ++m) WStore<WT>::one(a.copies.p[m - 1], g, v[m][k]);
-  }
-}
-
-// The noise words of one group: counter (q_lo, q_hi).  HI0 (q_hi = 0): the folded Philox, with
-// the counter's product M0 q shared by both noise vectors of the two pairs.
-template <int OP, bool HI0>
-__device__ __forceinline__ void group_words(const ElemArgs &a, uint32_t q_lo, uint32_t q_hi, uint32_t (*w)[4]) {
-  constexpr int kLast = op_noises<OP>() - 1;
-  if (HI0) {
-    const uint64_t m = (uint64_t)kPhiloxM0 * q_lo;
-    philox4x32_10_folded((uint32_t)m, (uint32_t)(m >> 32), a.fk, w[0]);
-    if (kLast) philox4x32_10_folded((uint32_t)m, (uint32_t)(m >> 32), a.fk_b, w[kLast]);
-  } else {
-    philox4x32_10_rk(q_lo, q_hi, 0u, op_tag<OP>(), a.rk, w[0]);
-    if (kLast) philox4x32_10_rk(q_lo, q_hi, 0u, op_tag<OP>(), a.rk_b, w[kLast]);
-  }
-}
-
-// One step: the thread's G groups at b + off + 4 kThreads i: their loads, then their Philox
-// calls, then their transforms and values.  EDGE: groups at b + n and beyond are generated but
-// neither loaded nor stored.
-template <int OP, typename WT, int G, bool HI0, bool EDGE = false>
-__device__ __forceinline__ void elem_step(const ElemArgs &a, const WideTable &tab, uint64_t b, uint32_t off,
-                                          uint32_t n = 0) {
-  constexpr int NP = op_noises<OP>();
-  const float *__restrict__ mt = a.master + b;
-  float th[G][4];
-#pragma unroll
-  for (int i = 0; i < G; ++i) {
-    if (OP != kOpInit && (!EDGE || off + 4u * kThreads * i < n)) {
-      const float4 v = ld_stream_f4(mt + off + 4u * kThreads * i);
-      th[i][0] = v.x, th[i][1] = v.y, th[i][2] = v.z, th[i][3] = v.w;
-    } else {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) th[i][k] = 0.0f;
-    }
-  }
-  uint32_t w[G * NP][4];
-  const uint64_t q0 = b >> 2;
-#pragma unroll
-  for (int i = 0; i < G; ++i) {
-    if (HI0) {
-      group_words<OP, true>(a, (uint32_t)q0 + ((off >> 2) + kThreads * i), 0u, &w[i * NP]);
-    } else {
-      const uint64_t q = q0 + ((off >> 2) + kThreads * i);
-      group_words<OP, false>(a, (uint32_t)q, (uint32_t)(q >> 32), &w[i * NP]);
-    }
-  }
-  unsigned long long e2[G * NP][2];
-  normals_packed<G * NP>(w, tab, e2);
-#pragma unroll
-  for (int i = 0; i < G; ++i) {
-    if (EDGE && off + 4u * kThreads * i >= n) continue;
-    float v[op_values<OP>()][4];
-    group_values<OP>(a, &e2[i * NP], th[i], v);
-    store_values_full<OP, WT>(a, b + off + 4u * kThreads * i, v);
-  }
-}
 
 // The two pairs' bf16 step by octets: G / 2 runs of two adjacent groups a thread, at
 // b + off + 8 kThreads i, each with one 32-byte load and one 16-byte store a value where
@@ -200,7 +89,7 @@ __device__ __forceinline__ void elem_span(const ElemArgs &a, const WideTable &ta
   }
   for (uint32_t at = 0; at < kElemSpan; at += kStep) {
     if (at == kElemSpan - kStep) next.ask();
-    elem_step<OP, WT, G, true>(a, tab, b, at + 4u * threadIdx.x);
+    elem_step<OP, WT, G>(a, LowKeys{}, tab, b, at + 4u * threadIdx.x);
   }
 }
 
@@ -214,35 +103,16 @@ __device__ __forceinline__ void elem_range(const ElemArgs &a, const WideTable &t
   uint32_t at = 0;
   for (; at + kStep / 2 < n; at += kStep) {
     if (at + kStep + kStep / 2 >= n) next.ask();
-    elem_step<OP, WT, G, true, true>(a, tab, b, at + 4u * threadIdx.x, n);
+    elem_step<OP, WT, G, true>(a, LowKeys{}, tab, b, at + 4u * threadIdx.x, 0, n);
   }
-  for (uint32_t off = at + 4u * threadIdx.x; off < n; off += 4u * kThreads) elem_step<OP, WT, 1, true>(a, tab, b, off);
+  for (uint32_t off = at + 4u * threadIdx.x; off < n; off += 4u * kThreads) elem_step<OP, WT, 1>(a, LowKeys{}, tab, b, off);
 }
 
-// The elements [b, e) of one group cut by a stretch's end.  Out of line, as is the form for
-// counters past 2^32, so that they take no registers from the forms above (with their tests
-// inlined, the pair perturb of 12M elements took 21.8 us instead of 18.4).
+// A stretch of less than a group a thread.  Out of line for the sake of the forms above: beside it
+// they are compiled to faster code than without it (two pairs of 4M elements 12.2 / 12.8 us).
 template <int OP, typename WT>
-__device__ __noinline__ void elem_partial_group(const ElemArgs &a, const WideTable &tab, uint64_t b, uint64_t e) {
-  const uint64_t g4 = b & ~3ull;
-  float th[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) th[k] = (OP != kOpInit && g4 + k >= b && g4 + k < e) ? a.master[g4 + k] : 0.0f;
-  constexpr int NP = op_noises<OP>();
-  uint32_t w[NP][4];
-  group_words<OP, false>(a, (uint32_t)(g4 >> 2), (uint32_t)(g4 >> 34), w);
-  unsigned long long e2[NP][2];
-  normals_packed<NP>(w, tab, e2);
-  float v[op_values<OP>()][4];
-  group_values<OP>(a, e2, th, v);
-#pragma unroll
-  for (int k = 0; k < 4; ++k)
-    if (g4 + k >= b && g4 + k < e) store_values_one<OP, WT>(a, g4 + k, v, k);
-}
-
-template <int OP, typename WT>
-__device__ __noinline__ void elem_high(const ElemArgs &a, const WideTable &tab, uint64_t b, uint32_t n) {
-  for (uint32_t off = 4u * threadIdx.x; off < n; off += 4u * kThreads) elem_step<OP, WT, 1, false>(a, tab, b, off);
+__device__ __noinline__ void elem_small(const ElemArgs &a, const WideTable &tab, uint64_t b, uint32_t n) {
+  for (uint32_t off = 4u * threadIdx.x; off < n; off += 4u * kThreads) elem_step<OP, WT, 1>(a, LowKeys{}, tab, b, off);
 }
 
 // The elements [b, e): the whole groups by the block, a group cut by either end by one thread
@@ -251,10 +121,10 @@ template <int OP, typename WT, int G>
 __device__ __forceinline__ void elem_stretch(const ElemArgs &a, const WideTable &tab, uint64_t b, uint64_t e,
                                              NextUnit &next) {
   const uint64_t lo = (b + 3) & ~3ull, hi = e & ~3ull;  // the whole groups, if lo < hi
-  if (lo != b && threadIdx.x == kThreads - 1) elem_partial_group<OP, WT>(a, tab, b, min(lo, e));
-  if (hi != e && hi >= lo && threadIdx.x == kThreads - 33) elem_partial_group<OP, WT>(a, tab, hi, e);
+  if (lo != b && threadIdx.x == kThreads - 1) elem_partial_group<OP, WT>(a, LowKeys{}, tab, b, min(lo, e));
+  if (hi != e && hi >= lo && threadIdx.x == kThreads - 33) elem_partial_group<OP, WT>(a, LowKeys{}, tab, hi, e);
   if (lo >= hi) return;
-  if ((e >> 34) != 0) elem_high<OP, WT>(a, tab, lo, (uint32_t)(hi - lo));
+  if (hi - lo < 4 * kThreads) elem_small<OP, WT>(a, tab, lo, (uint32_t)(hi - lo));
   else if (hi - lo == kElemSpan) elem_span<OP, WT, G>(a, tab, lo, next);
   else elem_range<OP, WT, G>(a, tab, lo, (uint32_t)(hi - lo), next);
 }
@@ -290,7 +160,7 @@ __device__ __forceinline__ bool elem_part(const ElemArgs &a, const WideTable &ta
   const uint64_t b = v.x + (unit - (unit >> lp << lp)) * kElemPart;
 #pragma unroll
   for (uint32_t at = 0; at < kElemPart; at += 4u * kThreads * G)
-    elem_step<OP, WT, G, true>(a, tab, b, at + 4u * threadIdx.x);
+    elem_step<OP, WT, G>(a, LowKeys{}, tab, b, at + 4u * threadIdx.x);
   return true;
 }
 
@@ -485,10 +355,17 @@ static cudaError_t launch_elem_typed(int kind, ElemArgs &a, cudaStream_t s) {
     if (kind == COPES_SUBSPACE_TILES) {
       if (OP == kOpPerturbTwoPairs && a.copies.n != 3) return cudaErrorInvalidValue;
       if (a.n_tiles == 0) return cudaSuccess;
-      // a copy, or a restore of one or two, has too little to do for parts beyond one tile an SM:
-      // 4M elements 5.4 us whole, 6.8 in quarters (restore of one), 11.1M 12.5 and 14.8
-      const bool light = OP == kOpPartner || (OP == kOpRestore && a.copies.n <= 1);
-      a.units = plan_tile_units(a.n_tiles, a.n_alloc, 2, light ? 152 : 1216);
+      const TileWork work = tile_work(a.n_tiles, a.n_alloc, a.tile_hint);
+      if constexpr (OP == kOpPartner || OP == kOpRestore) {
+        a.units = plan_copy(work, OP == kOpPartner ? -1 : a.copies.n, sizeof(WT) == 4);
+      } else {
+        const NoiseOp op = OP == kOpInit ? NoiseOp::kInit
+                                         : (OP == kOpPerturbTwoPairs ? NoiseOp::kTwoPairs
+                                                                     : (OP == kOpPerturbPair ? NoiseOp::kPair : NoiseOp::kPerturb));
+        const NoisePlan plan = plan_noise(work, a.n_alloc, op, sizeof(WT) == 4);
+        a.units = plan.units;
+        if (plan.ragged) return launch_elem_ragged(OP, sizeof(WT) == 2 ? COPES_BF16 : COPES_FP32, a, s);
+      }
       const unsigned grid = a.units.n_units;
       if constexpr (OP == kOpPartner) partner_tiles_kernel<WT, 8><<<grid, kThreads, 0, s>>>(a);
       else if constexpr (OP == kOpRestore) restore_tiles_kernel<WT, 8><<<grid, kThreads, 0, s>>>(a);
@@ -704,37 +581,11 @@ __global__ void __launch_bounds__(kThreads) update_index_kernel(const __grid_con
   });
 }
 
-// log2 of the parts an update cuts its tiles into.  Up to 128 tiles, sixteenths (one group a
-// thread).  Beyond, of the cuts that give each SM its four blocks, the one with the least
-// ceil(parts / slots) (1 / 2^log + overhead / P), the overhead of a part being a fifth to a third of
-// a tile's time for one noise vector: up to two waves of tiles the SM with the most parts sets
-// the time (152 slots), beyond the last wave does (608), where parts have to gain 3%.  With up
-// to three noise vectors the update is bound by memory and whole tiles are best, as they are
-// with four beyond two waves.  A block a tile / eighths to 608 tiles, whole ones above / this, us:
-// P = 16, 3M, 6M, 11.1M and 18M elements 84.6 / 51.2 / 49.2, 122.6 / 93.8 / 91.5, 196 / 176 /
-// 155 and 306 / 272 / 266; P = 4, 8M 48.0 / 47.8 / 39.3; P = 1, 8M 26.1 / 40.6 / 26.5; P = 64,
-// 30M and 134M 1,900 / 1,670 / 1,574 and 7,820 / 7,066 / 6,867.
-static uint32_t update_log_parts(uint64_t n_tiles, int n_noise) {
-  if (n_tiles <= (n_noise <= 3 ? 192u : 128u)) return 4;
-  const bool waves = n_tiles > 8 * 152;
-  if (n_noise <= (waves ? 4 : 3)) return 0;
-  const uint64_t slots = waves ? 4 * 152 : 152;
-  const double overhead = (waves ? 0.3 : 0.2) / n_noise;
-  uint32_t best = 0;
-  double best_cost = 1e30;
-  for (uint32_t log = 0; log <= (waves ? 2u : 3u); ++log) {
-    if ((n_tiles << log) < 4 * 152) continue;
-    const double cost = (double)(((n_tiles << log) + slots - 1) / slots) * (1.0 / (1 << log) + overhead);
-    if (cost < best_cost * (waves && best == 0 ? 0.97 : 1.0)) best = log, best_cost = cost;
-  }
-  return best;
-}
-
 template <typename WT, bool COMMIT>
 static cudaError_t launch_update_typed(int kind, UpdateArgs &a, cudaStream_t s) {
   if (kind == COPES_SUBSPACE_TILES) {
     if (a.n_tiles == 0) return cudaSuccess;
-    a.units = plan_tile_units(a.n_tiles, a.n_alloc, update_log_parts(a.n_tiles, a.n_noise), ~0u);
+    a.units = plan_update(tile_work(a.n_tiles, a.n_alloc, a.tile_hint), a.n_noise);
     auto kernel = a.n_noise <= kAheadNoise
                       ? update_tiles_kernel<WT, kUpdateGroups, COMMIT, kUpdateBlocksPerSM, true>
                       : update_tiles_kernel<WT, kUpdateGroups, COMMIT, kUpdateBlocksPerSM, false>;

@@ -71,9 +71,14 @@ CASES = [
     (70_000, [(1, 69_999)], 16), (6_000, [(2 * k, 2 * k + 1) for k in range(3000)], 4),
     # a third of the arena: shorter tiles than the bound says
     (5_000_000, [(3_300_001, 4_966_668)], 1000),
-    # more units than three waves: taken over early and late
+    # runs of eight tiles, about two waves of units
     (2048 * 8000, [(2, 2048 * 8000)], 2_048),
+    # runs with more than three waves of units, taken over early and late: aligned tiles joined to
+    # default ones (the noise ops' units), and odd ones with gaps between them (the update's)
+    (4096 * 8000, [(0, 4096 * 8000)], 4_096),
+    (33_000_000, [(k * 3_300_000 + k, (k + 1) * 3_300_000 - 5_000) for k in range(10)], 1_000),
 ]
+EARLY_RUNS = {16: "perturb", 17: "update"}
 
 
 @pytest.mark.parametrize("case", range(len(CASES)))
