@@ -1,6 +1,6 @@
 // Partition replay (Supp. A.8 "Partition Replay"; Eq. 7): the ES kernels over subspace k
 // of the hash partition (K, seed) with membership recomputed from the partition seed, not
-// read from a stored index list.  Each block takes 4 consecutive 16,384-element hash
+// read from a stored index list.  Each block takes 1 to 4 consecutive 16,384-element hash
 // tiles; each warp streams through its 2,048-element stretch of every tile (replay_stream):
 //  - it hashes 32 four-element groups at a time -- one Philox4x32-10 call per group at
 //    counter (e >> 2, tensor id, TAG_PARTITION), bucket floor(x K / 2^32) per word, or,
@@ -82,7 +82,7 @@ __device__ __forceinline__ void replay_stream(const ReplayArgs &r, uint64_t n_al
   constexpr int U = BATCH / 32;
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t warp = threadIdx.x >> 5;
-  const uint64_t per_block = (r.n_tiles + gridDim.x - 1) / gridDim.x;  // as replay_blocks chose
+  const uint64_t per_block = (r.n_tiles + gridDim.x - 1) / gridDim.x;  // at most what replay_blocks took
   const uint64_t t_first = blockIdx.x * per_block;
   const uint64_t t_end = min(t_first + per_block, r.n_tiles);
   // buffer entries are (tile within the block) << 16 | (offset within the tile); each warp
@@ -183,22 +183,32 @@ static __device__ __noinline__ uint32_t replay_word_high(const ElemArgs &a, uint
   return replay_word<OP>(a, g);
 }
 
-// Perturb / restore / commit / init over the members of the block's hash tiles: four
+// Perturb / restore / commit / init over the members of the block's hash tiles: BATCH / 32
 // members per lane per batch, their master loads issued together.  The hashing variant is
 // bound by its instructions: a batch's noise is formed together, from one word of a Philox
-// block each, whether or not a member is to be stored (perturb of 16.8M members of 2^28
-// elements 370 -> 336 us).  The mask variant is bound by scattered sectors and keeps fewer
-// registers instead (pair 373 us, 378 with single words).
-template <int OP, typename WT, bool MASK>
+// block each (perturb of 16.8M members of 2^28 elements 370 -> 336 us).  The mask variant is
+// bound by scattered sectors and keeps fewer registers instead (pair 373 us, 378 with single
+// words).
+//
+// Batches of 128, but 64 for the hashing pair of sparse subspaces: a warp's stretch then has about
+// one batch or none, what is left over is processed by the block one or two at a time, and
+// more warps fit an SM (38 registers for 56).  Pair of 200M elements, 128 / 64: bf16 K = 2 615 /
+// 636 us, K = 4 420 / 426, K = 16 278 / 275, K = 64 240 / 227; fp32 K = 16 343 / 358, K = 64 242 / 227.
+// The pool's places that hold no member form no noise, where the test costs no more than it
+// saves: not in the fp32 pair of dense subspaces and in init (45M, K = 2: 172 / 179 and 160 / 173).
+template <typename WT>
+constexpr int sparse_k() { return sizeof(WT) == 2 ? 16 : 32; }
+
+template <int OP, typename WT, bool MASK, int BATCH>
 __global__ void __launch_bounds__(kThreads) replay_elem_kernel(const __grid_constant__ ElemArgs a,
                                                                const __grid_constant__ ReplayArgs r) {
-  constexpr int BATCH = 128;
   constexpr int U = BATCH / 32;
   __shared__ uint32_t s_buf[kThreads / 32][BATCH + 128];
   __shared__ uint32_t s_pool[(kThreads / 32) * BATCH];
   __shared__ uint64_t s_g0[kThreads / 32][kReplayTilesPerBlock];
   __shared__ int s_pool_n;
   constexpr bool kNoise = OP != kOpRestore && OP != kOpPartner;
+  constexpr bool kSkip = OP == kOpPerturb || (OP == kOpPerturbPair && (BATCH == 64 || sizeof(WT) == 2));
   __shared__ __align__(16) float4 s_tab[kNoise ? SlimTable::kFloat4s : 1];
   if (threadIdx.x == 0) s_pool_n = 0;
   if (kNoise) SlimTable::fill(s_tab);
@@ -224,6 +234,7 @@ __global__ void __launch_bounds__(kThreads) replay_elem_kernel(const __grid_cons
       uint32_t wd[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
+        if (kSkip && !ok_in[u]) continue;  // known when compiled but for the pool
         const uint64_t m = (uint64_t)kPhiloxM0 * (uint32_t)(g[u] >> 2);
         const bool h = (uint32_t)g[u] & 2u, odd = (uint32_t)g[u] & 1u;
         wd[u] = a.n_alloc > 1ull << 34
@@ -232,7 +243,10 @@ __global__ void __launch_bounds__(kThreads) replay_elem_kernel(const __grid_cons
                                          h ? a.rk[19] : a.rk[18]);
       }
 #pragma unroll
-      for (int u = 0; u < U; u += 2) unpack_f32x2(normal_pair(wd[u], wd[u + 1], tab), eps[u], eps[u + 1]);
+      for (int u = 0; u < U; u += 2) {
+        if (kSkip && !ok_in[u]) continue;  // then u + 1 is not either
+        unpack_f32x2(normal_pair(wd[u], !kSkip || ok_in[u + 1] ? wd[u + 1] : 0u, tab), eps[u], eps[u + 1]);
+      }
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -292,9 +306,18 @@ __global__ void __launch_bounds__(kThreads) replay_update_kernel(const __grid_co
 // Tiles per block: 4, whose members share the pool of leftovers, while that leaves 608 blocks;
 // fewer below, where SMs would be idle: K = 4, 1M and 11.1M elements, perturb 34.6 -> 9.3 and 48.4 ->
 // 28.4 us, update (P = 16) 180 -> 51 and 262 -> 165 (4 / these).
-static unsigned replay_blocks(uint64_t n_tiles) {
-  const uint64_t per = std::min<uint64_t>(std::max<uint64_t>(n_tiles / 608, 1), kReplayTilesPerBlock);
+static unsigned replay_blocks(uint64_t n_tiles, uint64_t per) {
+  per = std::min<uint64_t>(std::max<uint64_t>(per, 1), kReplayTilesPerBlock);
   return (unsigned)((n_tiles + per - 1) / per);
+}
+static unsigned replay_elem_blocks(uint64_t n_tiles) { return replay_blocks(n_tiles, n_tiles / 608); }
+
+// The update's blocks also fill a table, and for few noise vectors that is much of their time: a
+// second wave of a few blocks costs more than fewer blocks do.  P = 1, K = 4, 16 and 64 in the
+// mean, 22M, 30M and 36M elements, tiles as above / one more, 55 / 49, 73 / 68 and 81 / 75 us; P = 4
+// and 16, K = 4, 24M 121 / 134 and 318 / 362.
+static unsigned replay_update_blocks(uint64_t n_tiles, int n_noise) {
+  return replay_blocks(n_tiles, n_tiles / 608 + (n_noise <= 2 && n_tiles >= 2 * 608 ? 1 : 0));
 }
 
 // Membership mask of subspace r.k: bit (e mod 32) of word tile * 512 + e / 32 is set when
@@ -334,10 +357,17 @@ cudaError_t launch_replay_mask(const ReplayArgs &r, uint64_t n_alloc, uint32_t *
 template <int OP, typename WT>
 static cudaError_t launch_replay_elem_typed(const ElemArgs &a, const ReplayArgs &r, cudaStream_t s) {
   if (r.n_tiles == 0) return cudaSuccess;
-  if (r.mask)
-    replay_elem_kernel<OP, WT, true><<<replay_blocks(r.n_tiles), kThreads, 0, s>>>(a, r);
-  else
-    replay_elem_kernel<OP, WT, false><<<replay_blocks(r.n_tiles), kThreads, 0, s>>>(a, r);
+  const unsigned blocks = replay_elem_blocks(r.n_tiles);
+  if (r.mask) {
+    replay_elem_kernel<OP, WT, true, 128><<<blocks, kThreads, 0, s>>>(a, r);
+    return cudaGetLastError();
+  }
+  if constexpr (OP == kOpPerturbPair)
+    if (r.K >= sparse_k<WT>()) {
+      replay_elem_kernel<OP, WT, false, 64><<<blocks, kThreads, 0, s>>>(a, r);
+      return cudaGetLastError();
+    }
+  replay_elem_kernel<OP, WT, false, 128><<<blocks, kThreads, 0, s>>>(a, r);
   return cudaGetLastError();
 }
 
@@ -368,7 +398,7 @@ static cudaError_t launch_replay_update_typed(const UpdateArgs &a, const ReplayA
   // 8.5 KB static
   const cudaError_t e = allow_smem((const void *)kernel, smem + 16 * 1024, gather_smem_bytes(COPES_MAX_NOISE));
   if (e != cudaSuccess) return e;
-  kernel<<<replay_blocks(r.n_tiles), kThreads, smem, s>>>(a, r);
+  kernel<<<replay_update_blocks(r.n_tiles, a.n_noise), kThreads, smem, s>>>(a, r);
   return cudaGetLastError();
 }
 

@@ -237,6 +237,24 @@ def test_hashing_past_counter_2_32_equals_the_mask(copes):
     copes.check()
 
 
+@pytest.mark.parametrize("K", [2, 15, 16, 31, 32, 64])
+def test_pairs_of_dense_and_sparse_subspaces_equal_the_lists(copes, K):
+    """The hashing pair takes its members in batches of 128, of sparse subspaces of 64; what is left
+    over is pooled, up to many times the block's threads."""
+    n, k = 5 * 16_384 - 777, 1
+    lay, theta = copes.Layout([n]), torch.randn(n, device="cuda")
+    for dtype in (torch.bfloat16, torch.float32):
+        out = []
+        for sub in (copes.hash_replay_partition(lay, K, 77)[k], copes.hash_partition(lay, K, 77)[k]):
+            a = copes.Arena(torch.zeros(n, dtype=dtype, device="cuda"), theta.clone())
+            buf = torch.zeros(n, dtype=dtype, device="cuda")
+            copes.perturb_pair(a, sub, 5, 1e-1, buf)
+            out.append((a.w, buf))
+        for x, y in zip(*out):
+            assert torch.equal(x, y)
+    copes.check()
+
+
 def test_updates_past_counter_2_32_equal_the_tiles(copes):
     """Index-list and replayed updates on both sides of index 2^34, element for element those
     over TILES (checked against the oracle there)."""
