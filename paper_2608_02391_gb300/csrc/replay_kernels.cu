@@ -219,6 +219,7 @@ __global__ void __launch_bounds__(kThreads) replay_elem_kernel(const __grid_cons
                              [&](const uint64_t (&g)[U], const bool (&ok_in)[U]) {
     bool ok[U];
     float th[U];
+    WT partner[U];  // of the partner copy: all loads before the first store
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       ok[u] = ok_in[u];
@@ -228,6 +229,7 @@ __global__ void __launch_bounds__(kThreads) replay_elem_kernel(const __grid_cons
         ok[u] = false;
       }
       th[u] = (OP != kOpInit && OP != kOpPartner && ok[u]) ? master[g[u]] : 0.0f;
+      if (OP == kOpPartner && ok[u]) partner[u] = reinterpret_cast<const WT *>(a.partner)[g[u] - a.partner_base];
     }
     float eps[U];
     if constexpr (kNoise && !MASK) {
@@ -252,7 +254,7 @@ __global__ void __launch_bounds__(kThreads) replay_elem_kernel(const __grid_cons
     for (int u = 0; u < U; ++u) {
       if (!ok[u]) continue;
       if constexpr (OP == kOpPartner) {
-        reinterpret_cast<WT *>(a.w)[g[u]] = reinterpret_cast<const WT *>(a.partner)[g[u] - a.partner_base];
+        reinterpret_cast<WT *>(a.w)[g[u]] = partner[u];
         continue;
       }
       float v, vp = 0.0f;
