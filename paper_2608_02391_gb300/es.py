@@ -115,7 +115,8 @@ def perturb_members(arena: copes.Arena, sub: copes.SubspaceHandle, members: Sequ
         perturb, pair, copy = copes.backup_perturb, copes.backup_perturb_pair, copes.backup_perturb_partner
     else:
         perturb, pair, copy = copes.perturb, copes.perturb_pair, copes.perturb_partner
-    nid, sign, seeds = np.asarray(nid).tolist(), np.asarray(sign).tolist(), [int(x) for x in seeds]
+    # element by element, an array is slower to read than the list of its values
+    nid, sign = (x.tolist() if isinstance(x, np.ndarray) else x for x in (nid, sign))
     two_pairs = partner is not None and partner.two_pairs and sub.kind == copes.SUBSPACE_TILES
     staged = None  # the member whose weights the partner buffer holds
     ready = {}     # member -> the working copy that already holds its weights
@@ -128,12 +129,12 @@ def perturb_members(arena: copes.Arena, sub: copes.SubspaceHandle, members: Sequ
         elif staged == i:
             _timed(events, "partner", copy, arena, sub, partner.buf, partner.base)
         else:
-            seed, ss = seeds[nid[i]], float(sign[i]) * s_k
+            seed, ss = int(seeds[nid[i]]), float(sign[i]) * s_k
             nxt = members[pos + 1] if partner is not None and pos + 1 < len(members) else None
             quad = members[pos:pos + 4] if two_pairs else ()
             if (len(quad) == 4 and _antithetic(nid, sign, quad[0], quad[1]) and _antithetic(nid, sign, quad[2], quad[3])
                     and sign[quad[2]] == sign[i]):
-                _timed(events, "perturb", copes.perturb_two_pairs, arena, sub, seed, seeds[nid[quad[2]]], ss)
+                _timed(events, "perturb", copes.perturb_two_pairs, arena, sub, seed, int(seeds[nid[quad[2]]]), ss)
                 ready = {quad[1]: arena.w2, quad[2]: arena.w3, quad[3]: arena.w4}
             elif nxt is not None and _antithetic(nid, sign, i, nxt):
                 _timed(events, "perturb", pair, arena, sub, seed, ss, partner.buf, partner.base)

@@ -108,3 +108,12 @@ def test_four_copies_on_a_slice_that_splits_the_groups(calls):
     seen = four_copy_run(range(3, 10), 12)
     assert [i for i, _ in seen] == list(range(3, 10))
     assert calls == [("perturb", 101, -0.5), ("two_pairs", 102, 103, 0.5), ("pair", 104, 0.5, 0)]
+
+
+def test_seeds_and_tables_of_any_kind_are_read_by_the_members_visited_only(calls):
+    """Seeds, noise ids and signs may be whatever can be indexed, and hold no more than the members
+    that are visited need."""
+    es.perturb_members(None, None, [2, 3, 5], {2: 1, 3: 1, 5: 2}, {2: 1, 3: -1, 5: -1}, {1: np.uint64(101), 2: 102}, 0.5,
+                       lambda i: None)
+    assert calls == [("perturb", 101, 0.5), ("perturb", 101, -0.5), ("perturb", 102, -0.5)]
+    assert all(type(seed) is int for _, seed, _ in calls)
