@@ -55,12 +55,13 @@ inline TileUnits cut_tiles(const TileWork &w, uint64_t unit) {
   return u;
 }
 
-// Whether the noise ops' kernels for default tiles serve these: aligned tiles of 4,096 elements,
-// or twice, four times ... as many, but for the last ones of their ranges.
+// Whether the noise ops' kernels for default tiles serve these: tiles of 4,096 elements, or twice,
+// four times ... as many, but for the last ones of their ranges, that begin with whole groups;
+// or so long that few of their parts do not.
 inline bool default_like(const TileWork &w) {
   uint64_t size = 4096;
   while (size < w.mean) size *= 2;
-  return w.aligned && 10 * w.mean > 9 * size;
+  return (w.aligned || size >= 4 * kDefaultTile) && 10 * w.mean > 9 * size;
 }
 
 // The noise ops over TILES, their kernel and its units.
@@ -95,7 +96,8 @@ inline NoisePlan plan_noise(const TileWork &w, uint64_t n_alloc, NoiseOp op, boo
   }
   if (n < 128u << 10) return NoisePlan{false, cut_tiles(w, 1024)};
   const bool pairs = op == NoiseOp::kPair || op == NoiseOp::kTwoPairs;
-  const uint64_t short_launch = op == NoiseOp::kInit ? 6u << 20 : kShortLaunch;
+  // parts of a tile with a cut group are whole spans only where they are as long as those
+  const uint64_t short_launch = !w.aligned ? 3u << 20 : (op == NoiseOp::kInit ? 6u << 20 : kShortLaunch);
   return NoisePlan{false, cut_tiles(w, n < short_launch || (fp32 && pairs) ? 4096 : kDefaultTile)};
 }
 

@@ -55,7 +55,8 @@ def test_the_mean_length_and_place_choose_the_kernel(plan):
     geometry = [((1000, 1000 * 16384, 1000 * 16384, 1), 0), ((1000, 1000 * 16384, 1000 * 16384, 0), 1),
                 ((1000, 1000 * 16384, 0, 0), 0), ((1000, 1 << 35, 1000 * 16384, 1), 1),
                 ((1000, 1 << 30, 1000 * 4096, 1), 0), ((1000, 1 << 30, 1000 * 1000, 1), 1),
-                ((1000, 1 << 30, 1000 * 6000, 1), 1), ((1000, 1 << 30, 1000 * 65_500, 1), 0)]
+                ((1000, 1 << 30, 1000 * 6000, 1), 1), ((1000, 1 << 30, 1000 * 65_500, 1), 0),
+                ((1000, 1 << 30, 1000 * 65_500, 0), 0)]
     for (_, ragged), plans in zip(geometry, plan([g for g, _ in geometry])):
         assert [p[0] for p in plans[:NOISE]] == [ragged] * NOISE
 
