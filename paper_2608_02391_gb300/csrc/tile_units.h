@@ -120,16 +120,18 @@ inline TileUnits plan_copy(const TileWork &w, int copies, bool fp32) {
 // 155 and 306 / 272 / 266; P = 4, 8M 48.0 / 47.8 / 39.3; P = 64, 30M and 134M 1,900 / 1,670 /
 // 1,574 and 7,820 / 7,066 / 6,867.
 // Up to three noise vectors the update is bound by memory and by its blocks' starts: the cut with
-// the least waves times its steps, a start counted as three of them.  P = 1, sixteenths to 192
-// tiles and whole ones above / this: 1M, 2M, 4M and 11.1M elements 6.5 / 5.1, 9.4 / 7.5, 12.2 /
-// 11.7 and 27.2 / 25.4.
+// the least waves times its steps, a start counted as three of them; beyond a wave of whole
+// tiles only for one noise vector, and where that gains a tenth.  Sixteenths to 192 tiles and whole
+// ones above / this, P = 1: 1M, 2M, 4M and 11.1M elements 6.5 / 5.1, 9.4 / 7.5, 12.2 / 11.7 and 27.2 /
+// 25.4; halves of 24M 44.0 / 46.8, and for P = 2 and 3 of 14.5M 36.2 / 38.2 and 47.1 / 49.7.
 inline uint32_t update_log_parts(uint64_t n_tiles, int n_noise) {
   uint32_t best = 0;
   double best_cost = 1e30;
   if (n_noise <= 3) {
     for (uint32_t log = 0; log <= 4; ++log) {
+      if (log && n_noise > 1 && n_tiles > kUnitsAtOnce) break;
       const double cost = (double)(((n_tiles << log) + kUnitsAtOnce - 1) / kUnitsAtOnce * ((16 >> log) + 3));
-      if (cost < best_cost) best = log, best_cost = cost;
+      if (cost < best_cost * (best == 0 && n_tiles > kUnitsAtOnce ? 0.9 : 1.0)) best = log, best_cost = cost;
     }
     return best;
   }
@@ -147,8 +149,7 @@ inline uint32_t update_log_parts(uint64_t n_tiles, int n_noise) {
 }
 
 // The run of short tiles that leaves the SM with the most units the least to do, as the cut of
-// default tiles: 11.1M elements in tiles of 1,000, P = 7 85 us in runs of 8, 77
-// in these.
+// default tiles: 11.1M elements in tiles of 1,000, P = 7 85 us in runs of 8, 77 in these.
 inline void best_run(TileUnits &u, const TileWork &w, int n_noise) {
   uint64_t best = ~0ull;
   for (uint32_t run = 1; run <= kRunMax && run * w.mean <= kDefaultTile + 1024; ++run) {
@@ -159,10 +160,26 @@ inline void best_run(TileUnits &u, const TileWork &w, int n_noise) {
   }
 }
 
+// The same for the parts of long tiles: 11.1M elements in tiles of 24,000, P = 6 85.6 us cut as
+// default tiles are, 74.1 in these.
+inline void best_parts(TileUnits &u, const TileWork &w, int n_noise) {
+  uint64_t best = ~0ull;
+  const uint64_t steps = (w.mean + 512) / 1024;
+  for (uint32_t log = 0; steps >> log >= 2; ++log) {
+    const uint64_t units = w.n_tiles << log;
+    if (units < kUnitsAtOnce) continue;
+    const uint64_t cost = (units + 151) / 152 * (((steps + (1u << log) - 1) >> log) * 1024 + 3277 / n_noise);
+    if (cost < best) best = cost, u.log_parts = log, u.n_units = (uint32_t)units;
+  }
+}
+
 inline TileUnits plan_update(const TileWork &w, int n_noise) {
   const uint64_t defaults = std::max<uint64_t>(w.elements() / kDefaultTile, 1);
   TileUnits u = cut_tiles(w, kDefaultTile >> update_log_parts(defaults, n_noise));
-  if (u.run > 1 && n_noise > 3 && defaults > 128 && defaults <= 2 * kUnitsAtOnce) best_run(u, w, n_noise);
+  if (n_noise > 3 && defaults > 128 && defaults <= 2 * kUnitsAtOnce) {
+    if (u.run > 1) best_run(u, w, n_noise);
+    else best_parts(u, w, n_noise);
+  }
   return u;
 }
 

@@ -78,3 +78,12 @@ def test_geometries_of_the_gpu_tests(plan):
         plans = plan([(n_tiles, n, sum(e - b for b, e in ranges), aligned)])[0]
         taken = plans[0] if which == "perturb" else plans[NOISE + COPIES]  # by up to three noise vectors
         assert not taken[0] and taken[3] > 1 and taken[1] > late + 100, (index, taken)
+
+
+@pytest.mark.parametrize("tile", [9_000, 12_000, 16_384, 20_000, 24_000, 50_000, 65_536])
+def test_an_update_of_a_few_waves_gives_every_sm_its_blocks(plan, tile):
+    for n in (2_200_000, 7_000_000, 11_111_112, 18_000_000):
+        n_tiles = -(-n // tile)
+        plans = plan([(n_tiles, n, n, 1)])[0]
+        for _, units, log, run in plans[NOISE + COPIES + 1:NOISE + COPIES + 3]:  # by 4 and 32 noise vectors
+            assert units >= 4 * 152 and run * tile >> log <= 2 * 16_384, (n, units, log, run)
