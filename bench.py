@@ -65,14 +65,14 @@ FALLBACK_HBM_GBS = 6800.0
 # subspaces of 2^28 parameters, where the writes still in L2 when the kernel ends are at most
 # 2% of its traffic.
 NCU_TRAFFIC = {
-    "perturb_two_pairs": {"kernel": "elem_tiles_kernel<perturb_two_pairs,bf16>", "source_sha": "0dc5faba317930d4",
-                          "bytes_per_elem": 11.945, "capture": "profiles/perturb_two_pairs_4b_slice.md",
+    "perturb_two_pairs": {"kernel": "elem_tiles_kernel<perturb_two_pairs,bf16>", "source_sha": "d2f3a63c2bcc6cb2",
+                          "bytes_per_elem": 11.941, "capture": "profiles/perturb_two_pairs_4b_slice.md",
                           "case": "two 2^28-parameter subspaces (--case 4b-slice-big)"},
-    "perturb_pair": {"kernel": "elem_tiles_kernel<perturb_pair,bf16>", "source_sha": "0dc5faba317930d4",
-                     "bytes_per_elem": 7.846, "capture": "profiles/perturb_pair_4b_slice.md",
+    "perturb_pair": {"kernel": "elem_tiles_kernel<perturb_pair,bf16>", "source_sha": "d2f3a63c2bcc6cb2",
+                     "bytes_per_elem": 7.847, "capture": "profiles/perturb_pair_4b_slice.md",
                      "case": "two 2^28-parameter subspaces (--case 4b-slice-big --weights dual)"},
-    "perturb": {"kernel": "elem_tiles_kernel<perturb,bf16>", "source_sha": "0dc5faba317930d4",
-                "bytes_per_elem": 5.876, "capture": "profiles/perturb_4b_slice.md",
+    "perturb": {"kernel": "elem_tiles_kernel<perturb,bf16>", "source_sha": "d2f3a63c2bcc6cb2",
+                "bytes_per_elem": 5.877, "capture": "profiles/perturb_4b_slice.md",
                 "case": "two 2^28-parameter subspaces (--case 4b-slice-big --weights single)"},
 }
 
@@ -165,7 +165,8 @@ def source_sha():
     dropped first, so an edit to a comment keeps a capture valid and any code change
     drops it."""
     h = hashlib.sha256()
-    for name in ("es_kernels.cu", "copes_device.cuh", "copes_internal.h", "es_common.cuh", "normal_coeffs.h"):
+    for name in ("es_kernels.cu", "elem_ops.cuh", "copes_device.cuh", "copes_internal.h", "es_common.cuh",
+                 "tile_units.h", "normal_coeffs.h"):
         with open(os.path.join(ROOT, "paper_2608_02391_gb300", "csrc", name)) as fh:
             text = re.sub(r"/\*.*?\*/", "", fh.read(), flags=re.S)
         text = re.sub(r"//[^\n]*", "", text)

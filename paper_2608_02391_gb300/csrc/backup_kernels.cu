@@ -101,7 +101,8 @@ __global__ void __launch_bounds__(kThreads, 8) backup_elem_kernel(const __grid_c
 // The update: all P noise vectors regenerated per group in registers (noise_sum_groups,
 // the tile update's loop), the backup read only after the noise loop, the new context
 // written to both copies.  Same launch shape as the tile update: G groups per thread,
-// 4 resident blocks per SM.  All counters of [b, e) have the high word s.q_hi.
+// 4 resident blocks per SM, and the same few spilled bytes.  All counters of [b, e) have the
+// high word s.q_hi.
 template <int G>
 __device__ __forceinline__ void backup_update_range(const UpdateArgs &a, uint16_t *backup, const UpdateSmem &s,
                                                     uint64_t b, uint64_t e) {

@@ -132,7 +132,9 @@ __device__ __forceinline__ void elem_stretch(const ElemArgs &a, const WideTable 
 // Groups per thread step, at 4 blocks of 256 threads per SM (64 registers).  Measured with
 // 16,384-element tiles on 2^28 elements (bf16; probe): the two-pairs perturb 2 groups
 // 0.509 ms, 1 group at 5 blocks 0.542 ms, 2 groups at 3 blocks 0.551 ms; the pair 4 groups
-// 0.311 ms, 2 groups at 5 or 6 blocks 0.320 and 0.314 ms.
+// 0.311 ms, 2 groups at 5 or 6 blocks 0.320 and 0.314 ms.  At 64 registers these kernels spill 20 to
+// 84 bytes a thread (most for the bf16 two pairs): about one local load a step of 16 normals and
+// 400 instructions, from L1; 3 blocks, which need none, are the slower.
 template <int OP>
 constexpr int elem_groups() { return OP == kOpPerturbTwoPairs ? 2 : 4; }
 
@@ -505,7 +507,8 @@ __device__ __forceinline__ void update_span(const UpdateArgs &a, const UpdateSme
 // Launch shape of the tile update: groups per thread and resident blocks per SM
 // (registers: 65536 / (256 x blocks) a thread).  Cycles per warp-normal at P = 16: 2 groups at
 // 4 blocks 33.1, at 5 blocks 32.9, at 3 blocks 33.2; 4 groups at 3 blocks 32.9; 1 group at 6
-// blocks 34.3.
+// blocks 34.3.  At 64 registers 48 to 56 bytes a thread spill, outside the noise loop: about one
+// local load a step (a warp's 256 elements) whatever P; at 3 blocks none do and it is no faster.
 constexpr int kUpdateGroups = 2;
 constexpr int kUpdateBlocksPerSM = 4;
 
