@@ -273,7 +273,7 @@ class SubspaceHandle:
             return self.replay
         if self.kind == SUBSPACE_TILES:
             return Subspace(SUBSPACE_TILES, self.tensor.data_ptr() if self.tensor.numel() else None,
-                            self.tensor.shape[0], None, max(self.numel, 0) << 1 | self.aligned)
+                            self.tensor.shape[0], None, max(int(self.numel or 0), 0) << 1 | bool(self.aligned))
         S = Subspace(SUBSPACE_INDICES, None, 0, self.tensor.data_ptr() if self.tensor.numel() else None,
                      self.tensor.numel())
         if self.gathered is not None:

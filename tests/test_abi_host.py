@@ -347,3 +347,12 @@ def test_backup_partner_arguments_are_rejected_before_any_launch(lib):
     assert lib.copes_backup_perturb_pair(ctypes.byref(p), ctypes.byref(s), 1, float("nan"), fake, 0, 1000,
                                          None) == copes.ERR_INVALID_ARG
     assert lib.copes_backup_perturb_partner(None, ctypes.byref(s), fake, 0, 1000, None) == copes.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("numel, said", [(None, 0), (0, 0), (-1, 0), (10, 10), (np.int64(10), 10), (10.0, 10)])
+@pytest.mark.parametrize("aligned", [True, False, np.bool_(False)])
+def test_a_tile_handle_says_what_it_knows_of_its_length(numel, said, aligned):
+    import torch
+    from paper_2608_02391_gb300 import copes
+    S = copes.SubspaceHandle(copes.SUBSPACE_TILES, torch.tensor([[0, 4], [4, 10]]), numel, aligned=aligned).struct()
+    assert (S.kind, S.n_tiles, S.n_index) == (copes.SUBSPACE_TILES, 2, said << 1 | bool(aligned))
